@@ -188,3 +188,18 @@ def test_kmeanspp_rejects_bad_draws(slk):
         slk.kmeanspp(X, 3, 10, [0.5, 0.5])
     with pytest.raises(slk.SlkError, match="INVALID_ARG"):
         slk.kmeanspp(X, 11, 0, [0.5] * 10)
+
+
+@pytest.mark.parametrize("N,D,L", [(255, 1, 9), (256, 3, 40), (257, 4, 40), (1000, 8, 60), (5000, 17, 300),
+                                   (3001, 36, 50), (3001, 64, 50), (2000, 132, 25), (400001, 12, 20)])
+@pytest.mark.parametrize("shift,scale", [(0.0, 1.0), (3e4, 1.0), (0.0, 1e-22), (0.0, 3e18)])
+def test_kmeanspp_screened_distances(slk, N, D, L, shift, scale):
+    """The bounds that skip float64 distances change no seed: lanes per point
+    4 to 32, tile edges, data far from the origin (the float32 distances are
+    coarse), and scales at which float32 squares underflow or overflow (the
+    bounds must step aside).  Index for index against the oracle."""
+    X, _ = inputs.blobs(N=N, D=D, n_blobs=8, centre_var=25.0, seed=N + D)
+    X = ((X + np.float32(shift)) * np.float32(scale)).astype(np.float32)
+    first, u = inputs.kmeanspp_draws(N, L, seed=D)
+    got = host(slk.kmeanspp(dev(X), L, first, u))
+    np.testing.assert_array_equal(got, oracle.kmeanspp(X, L, first, u))
