@@ -47,6 +47,19 @@ slk_status ensure_ws(slk_ctx* ctx, size_t bytes) {
     return SLK_OK;
 }
 
+slk_status ensure_ws_of(slk_ctx* ctx, size_t want, size_t least, bool* full) {
+    *full = true;
+    if (want <= ctx->ws_bytes) return SLK_OK;
+    if (want < ctx->ws_refused) {
+        const slk_status r = ensure_ws(ctx, want);
+        if (r != SLK_ERR_OOM) return r;
+        ctx->ws_refused = want;
+        ctx->err.clear();
+    }
+    *full = false;
+    return ensure_ws(ctx, least);
+}
+
 static cudaEvent_t take_event(slk_ctx* ctx) {
     if (!ctx->pool.empty()) {
         cudaEvent_t e = ctx->pool.back();
@@ -265,10 +278,12 @@ extern "C" slk_status slk_knn_graph(slk_ctx* ctx, const float* X, int64_t N, int
     CHECK_ARG(affinity == SLK_AFFINITY_BINARY || affinity == SLK_AFFINITY_HEAT, "bad affinity %d", affinity);
     CHECK_ARG(precision == SLK_KNN_FP32 || precision == SLK_KNN_BF16_RERANK, "bad precision %d", precision);
     CHECK_ARG(affinity != SLK_AFFINITY_HEAT || (w && sigma > 0.f), "HEAT needs w and sigma > 0");
-    slk_status r = ensure_ws(ctx, knn_ws_bytes(ctx, N, D, k, precision));
+    const size_t kb = knn_ws_bytes(ctx, N, D, k, precision), kb0 = knn_ws_min_bytes(ctx, N, D, k, precision);
+    bool full;
+    slk_status r = ensure_ws_of(ctx, kb, kb0, &full);
     if (r != SLK_OK) return r;
     DevState* st = dstate(ctx);
-    r = knn_graph_launch(ctx, X, N, D, k, precision, row_ptr, col_idx, dist2, ctx->ws, st);
+    r = knn_graph_launch(ctx, X, N, D, k, precision, row_ptr, col_idx, dist2, ctx->ws, full ? kb : kb0, st);
     if (r != SLK_OK) return r;
     if (w) {
         if (affinity == SLK_AFFINITY_HEAT) {
@@ -456,6 +471,7 @@ struct SolveBufs {
     float* w;
     float* mode_key;
     void* knn_ws;
+    size_t knn_bytes;
     // symmetric affinity (symmetrize): CSR of (K + K^t) / 2 and its scratch
     int64_t* srow_ptr;
     int32_t* scol;
@@ -463,13 +479,16 @@ struct SolveBufs {
     void* sym_ws;
 };
 
-size_t solve_ws_bytes(const slk_ctx* ctx, int64_t N, int D, int L, int k, const slk_params& p) {
+// knn_bytes: the graph's scratch (knn_ws_bytes, or knn_ws_min_bytes where that
+// much memory cannot be had).
+size_t solve_ws_bytes(const slk_ctx* ctx, int64_t N, int D, int L, int k, const slk_params& p,
+                      size_t knn_bytes) {
     size_t b = 0;
     b += 2 * align_up(sizeof(float) * (size_t)N * L, 256);
     b += 3 * align_up(sizeof(float) * (size_t)N * k, 256);
     b += align_up(sizeof(int64_t) * (size_t)(N + 1), 256);
     b += align_up(sizeof(float) * (size_t)L, 256);
-    b += knn_ws_bytes(ctx, N, D, k, p.knn_precision) + 512;
+    b += knn_bytes + 512;
     if (p.refine_init) b += init_modes_ws_bytes(ctx, N, D, L) + 512;
     if (p.symmetrize)
         b += align_up(sizeof(int64_t) * (size_t)(N + 1), 256) +
@@ -482,7 +501,7 @@ size_t solve_ws_bytes(const slk_ctx* ctx, int64_t N, int D, int L, int k, const 
 }
 
 SolveBufs carve_solve(WsCarver& wc, const slk_ctx* ctx, int64_t N, int D, int L, int k,
-                      const slk_params& p) {
+                      const slk_params& p, size_t knn_bytes) {
     SolveBufs b{};
     b.A = wc.take<float>((size_t)N * L);
     b.Zp = wc.take<float>((size_t)N * L);
@@ -491,7 +510,8 @@ SolveBufs carve_solve(WsCarver& wc, const slk_ctx* ctx, int64_t N, int D, int L,
     b.w = wc.take<float>((size_t)N * k);
     b.row_ptr = wc.take<int64_t>((size_t)N + 1);
     b.mode_key = wc.take<float>((size_t)L);
-    b.knn_ws = wc.take<unsigned char>(knn_ws_bytes(ctx, N, D, k, p.knn_precision));
+    b.knn_ws = wc.take<unsigned char>(knn_bytes);
+    b.knn_bytes = knn_bytes;
     b.init_ws = p.refine_init ? wc.take<unsigned char>(init_modes_ws_bytes(ctx, N, D, L)) : nullptr;
     if (p.symmetrize) {
         b.srow_ptr = wc.take<int64_t>((size_t)N + 1);
@@ -512,6 +532,18 @@ SolveBufs carve_solve(WsCarver& wc, const slk_ctx* ctx, int64_t N, int D, int L,
         b.loc_ws = wc.take<unsigned char>(locality_ws_bytes(N, L));
     }
     return b;
+}
+
+// Workspace of a solve and `more` bytes; *knn_bytes receives the graph's share.
+slk_status ensure_solve_ws(slk_ctx* ctx, int64_t N, int D, int L, int k, const slk_params& p, size_t more,
+                           size_t* knn_bytes) {
+    const size_t kb = knn_ws_bytes(ctx, N, D, k, p.knn_precision);
+    const size_t kb0 = knn_ws_min_bytes(ctx, N, D, k, p.knn_precision);
+    bool full;
+    const slk_status r = ensure_ws_of(ctx, solve_ws_bytes(ctx, N, D, L, k, p, kb) + more,
+                                      solve_ws_bytes(ctx, N, D, L, k, p, kb0) + more, &full);
+    *knn_bytes = full ? kb : kb0;
+    return r;
 }
 
 slk_status check_solve_args(slk_ctx* ctx, const float* X, int64_t N, int32_t D, int32_t L, int32_t k,
@@ -539,7 +571,7 @@ slk_status solve_device(slk_ctx* ctx, const float* X, int64_t N, int32_t D, int3
     DevState* st = dstate(ctx);
     cudaStream_t s = ctx->stream;
     slk_status r = knn_graph_launch(ctx, X, N, D, k, p.knn_precision, b.row_ptr, b.col_idx, b.dist2,
-                                    b.knn_ws, st);
+                                    b.knn_ws, b.knn_bytes, st);
     if (r != SLK_OK) return r;
     r = (sigma > 0.f) ? set_sigma_launch(ctx, sigma, st)
                       : sigma_launch(ctx, b.dist2, N * (int64_t)k, p.sigma_rule, st);
@@ -655,10 +687,11 @@ extern "C" slk_status slk_solve(slk_ctx* ctx, const float* X, int64_t N, int32_t
     if (params) p = *params; else slk_default_params(&p);
     slk_status r = check_solve_args(ctx, X, N, D, L, k, init_modes, p, Z, labels, modes, false);
     if (r != SLK_OK) return r;
-    r = ensure_ws(ctx, solve_ws_bytes(ctx, N, D, L, k, p));
+    size_t kb;
+    r = ensure_solve_ws(ctx, N, D, L, k, p, 0, &kb);
     if (r != SLK_OK) return r;
     WsCarver wc(ctx->ws);
-    const SolveBufs b = carve_solve(wc, ctx, N, D, L, k, p);
+    const SolveBufs b = carve_solve(wc, ctx, N, D, L, k, p, kb);
     return solve_device(ctx, X, N, D, L, k, lambda, sigma, init_modes, p, Z, labels, modes, stats, b);
 }
 
@@ -671,10 +704,12 @@ extern "C" slk_status slk_solve_host(slk_ctx* ctx, const float* X, int64_t N, in
     if (params) p = *params; else slk_default_params(&p);
     slk_status r = check_solve_args(ctx, X, N, D, L, k, init_modes, p, Z, labels, modes, true);
     if (r != SLK_OK) return r;
-    size_t need = solve_ws_bytes(ctx, N, D, L, k, p);
-    need += align_up(sizeof(float) * (size_t)N * D, 256) + align_up(sizeof(float) * (size_t)N * L, 256) +
-            align_up(sizeof(int32_t) * (size_t)N, 256) + 2 * align_up(sizeof(int32_t) * (size_t)L, 256) + 1024;
-    r = ensure_ws(ctx, need);
+    const size_t copies = align_up(sizeof(float) * (size_t)N * D, 256) +
+                          align_up(sizeof(float) * (size_t)N * L, 256) +
+                          align_up(sizeof(int32_t) * (size_t)N, 256) +
+                          2 * align_up(sizeof(int32_t) * (size_t)L, 256) + 1024;
+    size_t kb;
+    r = ensure_solve_ws(ctx, N, D, L, k, p, copies, &kb);
     if (r != SLK_OK) return r;
     WsCarver wc(ctx->ws);
     float* dX = wc.take<float>((size_t)N * D);
@@ -682,7 +717,7 @@ extern "C" slk_status slk_solve_host(slk_ctx* ctx, const float* X, int64_t N, in
     int32_t* dlab = wc.take<int32_t>((size_t)N);
     int32_t* dinit = wc.take<int32_t>((size_t)L);
     int32_t* dmodes = wc.take<int32_t>((size_t)L);
-    const SolveBufs b = carve_solve(wc, ctx, N, D, L, k, p);
+    const SolveBufs b = carve_solve(wc, ctx, N, D, L, k, p, kb);
     cudaStream_t s = ctx->stream;
     {
         PhaseScope ps(ctx, SLK_PHASE_TRANSFER);
@@ -861,14 +896,16 @@ extern "C" slk_status slk_solve_ms(slk_ctx* ctx, const float* X, int64_t N, int3
     if (r != SLK_OK) return r;
     CHECK_ARG(D <= SLK_MS_MAX_D, "D=%d must be <= %d", D, SLK_MS_MAX_D);
     CHECK_ARG(p.max_ms >= 1, "max_ms must be >= 1");
-    r = ensure_ws(ctx, solve_ws_bytes(ctx, N, D, L, k, p) + ms_bufs_bytes(ctx, N, D, L) + 1024);
+    size_t kb;
+    r = ensure_solve_ws(ctx, N, D, L, k, p, ms_bufs_bytes(ctx, N, D, L) + 1024, &kb);
     if (r != SLK_OK) return r;
     WsCarver wc(ctx->ws);
-    const SolveBufs b = carve_solve(wc, ctx, N, D, L, k, p);
+    const SolveBufs b = carve_solve(wc, ctx, N, D, L, k, p, kb);
     const MsBufs mb = carve_ms(wc, ctx, N, D, L);
     DevState* st = dstate(ctx);
     cudaStream_t s = ctx->stream;
-    r = knn_graph_launch(ctx, X, N, D, k, p.knn_precision, b.row_ptr, b.col_idx, b.dist2, b.knn_ws, st);
+    r = knn_graph_launch(ctx, X, N, D, k, p.knn_precision, b.row_ptr, b.col_idx, b.dist2, b.knn_ws,
+                         b.knn_bytes, st);
     if (r != SLK_OK) return r;
     r = (sigma > 0.f) ? set_sigma_launch(ctx, sigma, st)
                       : sigma_launch(ctx, b.dist2, N * (int64_t)k, p.sigma_rule, st);

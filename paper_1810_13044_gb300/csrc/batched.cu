@@ -501,11 +501,12 @@ extern "C" slk_status slk_solve_batched(slk_ctx* ctx, const slk_instance* inst, 
                            b, (long long)q.N, q.D, q.L, q.k);
     }
     // ---- workspace: per instance graph + A + Zs; shared kNN scratch; tables
-    size_t knn_max = 0;
+    size_t knn_max = 0, knn_least = 0;
     int64_t rows_total = 0, z_total = 0, nnz_total = 0, L_total = 0, ntiles = 0, nutiles = 0;
     for (int b = 0; b < count; ++b) {
         const slk_instance& q = inst[b];
         knn_max = std::max(knn_max, knn_ws_bytes(ctx, q.N, q.D, q.k, p.knn_precision));
+        knn_least = std::max(knn_least, knn_ws_min_bytes(ctx, q.N, q.D, q.k, p.knn_precision));
         rows_total += q.N;
         z_total += q.N * q.L;
         nnz_total += q.N * q.k;
@@ -515,7 +516,7 @@ extern "C" slk_status slk_solve_batched(slk_ctx* ctx, const slk_instance* inst, 
         nutiles += (q.N + 31) / 32;
     }
     constexpr int kAux = 8;   // graphs of different instances are built on kAux streams
-    size_t need = kAux * (align_up(knn_max, 256) + align_up(sizeof(DevState), 256)) + 4096;
+    size_t need = kAux * align_up(sizeof(DevState), 256) + 4096;
     need += count * (align_up(sizeof(int64_t) * 1, 256));  // slack
     need += align_up(sizeof(int64_t) * (rows_total + count), 256);
     need += 3 * align_up(sizeof(float) * nnz_total, 256) + align_up(sizeof(int32_t) * nnz_total, 256);
@@ -526,8 +527,11 @@ extern "C" slk_status slk_solve_batched(slk_ctx* ctx, const slk_instance* inst, 
     need += align_up(sizeof(unsigned) * 3 * count, 256) + 6 * align_up(sizeof(int) * count, 256);
     need += 2 * align_up(sizeof(double) * count, 256) + align_up(sizeof(float) * count, 256);
     need += (size_t)count * 8 * 256 + 64 * 256;   // alignment of the per-instance slices
-    slk_status r = ensure_ws(ctx, need);
+    bool full;
+    slk_status r = ensure_ws_of(ctx, need + kAux * align_up(knn_max, 256),
+                                need + kAux * align_up(knn_least, 256), &full);
     if (r != SLK_OK) return r;
+    if (!full) knn_max = knn_least;
     WsCarver wc(ctx->ws);
     void* knn_ws[kAux];
     DevState* aux_st[kAux];
@@ -598,7 +602,7 @@ extern "C" slk_status slk_solve_batched(slk_ctx* ctx, const slk_instance* inst, 
         moff += q.L;
         // the instance's graph and kernel width (same kernels as slk_solve)
         r = knn_graph_launch(ctx, q.X, q.N, q.D, q.k, p.knn_precision, row_ptr, col, dist2,
-                             knn_ws[lane_s], st);
+                             knn_ws[lane_s], knn_max, st);
         if (r != SLK_OK) { ctx->stream = s; return r; }
         r = (q.sigma > 0.f) ? set_sigma_launch(ctx, q.sigma, st)
                             : sigma_launch(ctx, dist2, q.N * (int64_t)q.k, p.sigma_rule, st);

@@ -27,6 +27,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "knn_group.cuh"
 #include "slk_internal.cuh"
 
 namespace {
@@ -108,33 +109,47 @@ __global__ void label_count_kernel(const int32_t* __restrict__ lab, int64_t N, i
     for (int l = threadIdx.x; l < L; l += blockDim.x) counts[(int64_t)blockIdx.x * L + l] = cnt[l];
 }
 
-// One block: base[b][l] = off[l] + sum_{b' < b} counts[b'][l]; off[L] = N.
-__global__ void label_scan_kernel(const int32_t* __restrict__ counts, int nb, int L,
-                                  int64_t* __restrict__ base, int64_t* __restrict__ off) {
-    __shared__ int64_t tot[SLK_MAX_L + 1];
-    for (int l = threadIdx.x; l < L; l += blockDim.x) {
-        int64_t s = 0;
-        for (int b = 0; b < nb; ++b) s += counts[(int64_t)b * L + l];
-        tot[l] = s;
+// Block l: base[b][l] = sum_{b' < b} counts[b'][l] and the label's total.
+__global__ void __launch_bounds__(256)
+label_scan_kernel(const int32_t* __restrict__ counts, int nb, int L, int64_t* __restrict__ base,
+                  int64_t* __restrict__ off) {
+    __shared__ int64_t wt[8];
+    const int l = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int per = (nb + 255) / 256, b0 = min(nb, t * per), b1 = min(nb, b0 + per);
+    int64_t s = 0;
+    for (int b = b0; b < b1; ++b) s += counts[(int64_t)b * L + l];
+    int64_t incl = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
     }
+    if (lane == 31) wt[w] = incl;
+    __syncthreads();
+    int64_t run = incl - s, all = 0;
+    for (int i = 0; i < 8; ++i) {
+        if (i < w) run += wt[i];
+        all += wt[i];
+    }
+    for (int b = b0; b < b1; ++b) {
+        base[(int64_t)b * L + l] = run;
+        run += counts[(int64_t)b * L + l];
+    }
+    if (t == 0) off[l] = all;
+}
+
+// off[l]: totals to first places; off[L] = N.
+__global__ void label_offsets_kernel(int L, int64_t* __restrict__ off) {
+    __shared__ int64_t tot[SLK_MAX_L];
+    for (int l = threadIdx.x; l < L; l += blockDim.x) tot[l] = off[l];
     __syncthreads();
     if (threadIdx.x == 0) {
         int64_t run = 0;
         for (int l = 0; l < L; ++l) {
-            const int64_t c = tot[l];
-            tot[l] = run;
             off[l] = run;
-            run += c;
+            run += tot[l];
         }
         off[L] = run;
-    }
-    __syncthreads();
-    for (int l = threadIdx.x; l < L; l += blockDim.x) {
-        int64_t run = tot[l];
-        for (int b = 0; b < nb; ++b) {
-            base[(int64_t)b * L + l] = run;
-            run += counts[(int64_t)b * L + l];
-        }
     }
 }
 
@@ -143,7 +158,8 @@ __global__ void label_scan_kernel(const int32_t* __restrict__ counts, int nb, in
 // increasing point order.  256 threads, one point per thread and round.
 __global__ void __launch_bounds__(256)
 label_scatter_kernel(const int32_t* __restrict__ lab, int64_t N, int L,
-                     const int64_t* __restrict__ base, int32_t* __restrict__ perm) {
+                     const int64_t* __restrict__ base, const int64_t* __restrict__ off,
+                     int32_t* __restrict__ perm) {
     extern __shared__ int sh[];
     int* run = sh;            // [L] placed so far in this block
     int* wc = sh + L;         // [8][L] per-warp counts of the round
@@ -163,7 +179,7 @@ label_scatter_kernel(const int32_t* __restrict__ lab, int64_t N, int L,
         if (ok) {
             int before = run[l];
             for (int ww = 0; ww < w; ++ww) before += wc[ww * L + l];
-            perm[base[(int64_t)blockIdx.x * L + l] + before + rin] = (int32_t)p;
+            perm[off[l] + base[(int64_t)blockIdx.x * L + l] + before + rin] = (int32_t)p;
         }
         __syncthreads();
         for (int ll = t; ll < L; ll += 256) {
@@ -515,13 +531,10 @@ slk_status init_modes_launch(slk_ctx* ctx, const float* X, int64_t N, int D, con
         SLK_LAUNCH_CHECK(ctx, "seed_assign_kernel");
     }
     // 2. stable counting sort by cluster
-    SLK_COUNT_LAUNCH(ctx, 3);
-    label_count_kernel<<<pl.nb, 256, sizeof(int) * L, s>>>(assign, N, L, counts);
-    label_scan_kernel<<<1, 256, 0, s>>>(counts, pl.nb, L, base, off);
-    label_scatter_kernel<<<pl.nb, 256, sizeof(int) * 9 * L, s>>>(assign, N, L, base, perm);
-    SLK_LAUNCH_CHECK(ctx, "counting sort");
+    slk_status r = label_sort_launch(ctx, assign, N, L, counts, base, off, perm);
+    if (r != SLK_OK) return r;
     // 3. centred operand and norms
-    slk_status r = knn_prep_fp32_launch(ctx, X, N, D, pl.Dp, pl.Np, colsum, mu, xt, norms, rho, st);
+    r = knn_prep_fp32_launch(ctx, X, N, D, pl.Dp, pl.Np, colsum, mu, xt, norms, rho, st);
     if (r != SLK_OK) return r;
     // 4. work items: every cluster's perm range cut into chunks (host, from the offsets)
     std::vector<int64_t> hoff(L + 1);
@@ -597,6 +610,21 @@ slk_status init_modes_launch(slk_ctx* ctx, const float* X, int64_t N, int D, con
     if (assign_out)
         SLK_CUDA_TRY(ctx, cudaMemcpyAsync(assign_out, assign, sizeof(int32_t) * N,
                                           cudaMemcpyDeviceToDevice, s));
+    return SLK_OK;
+}
+
+// Stable counting sort of the points by label: perm lists them, off the first
+// place of every label.
+slk_status label_sort_launch(slk_ctx* ctx, const int32_t* lab, int64_t N, int L, int32_t* counts,
+                             int64_t* base, int64_t* off, int32_t* perm) {
+    cudaStream_t s = ctx->stream;
+    const int nb = (int)((N + kSortChunk - 1) / kSortChunk);
+    SLK_COUNT_LAUNCH(ctx, 4);
+    label_count_kernel<<<nb, 256, sizeof(int) * L, s>>>(lab, N, L, counts);
+    label_scan_kernel<<<L, 256, 0, s>>>(counts, nb, L, base, off);
+    label_offsets_kernel<<<1, 256, 0, s>>>(L, off);
+    label_scatter_kernel<<<nb, 256, sizeof(int) * 9 * L, s>>>(lab, N, L, base, off, perm);
+    SLK_LAUNCH_CHECK(ctx, "counting sort");
     return SLK_OK;
 }
 
@@ -705,11 +733,10 @@ slk_status locality_perm_launch(slk_ctx* ctx, const float* A, int64_t N, int L, 
     int32_t* counts = wc.take<int32_t>((size_t)nb * L);
     int64_t* base = wc.take<int64_t>((size_t)nb * L);
     int64_t* off = wc.take<int64_t>(L + 1);
-    SLK_COUNT_LAUNCH(ctx, 5);
+    SLK_COUNT_LAUNCH(ctx, 2);
     row_argmax_kernel<<<grid_for(ctx, N, 256), 256, 0, s>>>(A, N, L, lab);
-    label_count_kernel<<<nb, 256, sizeof(int) * L, s>>>(lab, N, L, counts);
-    label_scan_kernel<<<1, 256, 0, s>>>(counts, nb, L, base, off);
-    label_scatter_kernel<<<nb, 256, sizeof(int) * 9 * L, s>>>(lab, N, L, base, perm);
+    const slk_status r = label_sort_launch(ctx, lab, N, L, counts, base, off, perm);
+    if (r != SLK_OK) return r;
     inverse_perm_kernel<<<grid_for(ctx, N, 256), 256, 0, s>>>(perm, N, inv);
     SLK_LAUNCH_CHECK(ctx, "locality order");
     return SLK_OK;

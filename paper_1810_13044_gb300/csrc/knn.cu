@@ -25,19 +25,14 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
-#include <algorithm>
 #include <stdint.h>
 
-#include "slk_internal.cuh"
+#include <algorithm>
 
-int knn_tc_tile_cols();
-int knn_tc_lists_per_split(int kc, int ew);
-slk_status knn_cand_split_launch(slk_ctx* ctx, const __nv_bfloat16* qh, const __nv_bfloat16* ql,
-                                 const float* qnorm, int64_t Fcap, const long long* rows_dev,
-                                 const __nv_bfloat16* xh, const __nv_bfloat16* xl,
-                                 const float* norms, int64_t N, int Dp, int64_t Np, int ew,
-                                 int splits, float* cand_d, int32_t* cand_i,
-                                 unsigned int* err_flag);
+#include "knn_cert.cuh"
+#include "knn_group.cuh"
+#include "knn_sweep.cuh"
+#include "slk_internal.cuh"
 
 namespace {
 
@@ -182,7 +177,8 @@ __device__ __forceinline__ void rho_kappa(float eh, float el, float vh, float vl
 // for every row.
 // aug (nullable, Np x 32 bfloat16): the folded-norm columns of the
 // tensor-core tiles, [1, 1, 1, a_p, 0...] in columns 0..15 and [a_p, 1, 1, 1,
-// 0...] in 16..31, a_p = (t1, t2, t3) the bfloat16 terms of -norms[p] / 2
+// 0...] in 16..31 (perm nullable: row p is point perm[p]; norms32 stays by
+// point), a_p = (t1, t2, t3) the bfloat16 terms of -norms[p] / 2
 // (t1 = bf16(x), t2 = bf16(x - t1), t3 = bf16(x - t1 - t2), each difference
 // exact in float32, so t1 + t2 + t3 is within 2^-24 (1.02) |x| of x); a
 // padding row has a_p = (-inf, 0, 0).
@@ -192,7 +188,8 @@ prep_rows_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
                  int64_t Np, const float* __restrict__ mu, int to_bf16,
                  float* __restrict__ xt32, __nv_bfloat16* __restrict__ xt16,
                  float* __restrict__ norms, float* __restrict__ rho,
-                 float* __restrict__ norms32, __nv_bfloat16* __restrict__ aug, DevState* st) {
+                 float* __restrict__ norms32, __nv_bfloat16* __restrict__ aug,
+                 const int32_t* __restrict__ perm, DevState* st) {
     __shared__ unsigned bmax_n, bmax_r, bmax_n32, bmax_k;
     if (threadIdx.x == 0) { bmax_n = 0u; bmax_r = 0u; bmax_n32 = 0u; bmax_k = 0u; }
     __syncthreads();
@@ -203,6 +200,7 @@ prep_rows_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
     unsigned my_n = 0u, my_r = 0u, my_n32 = 0u, my_k = 0u;
     for (int64_t p = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); p < Np;
          p += nw) {
+        const int64_t src = (perm && p < N) ? (int64_t)perm[p] : p;
         float n2v[V], e2v[V], v2v[V];
 #pragma unroll
         for (int q = 0; q < V; ++q) { n2v[q] = 0.f; e2v[q] = 0.f; v2v[q] = 0.f; }
@@ -213,11 +211,11 @@ prep_rows_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
             for (int q = 0; q < V; ++q) v[q] = 0.f;
             if (p < N && j < D) {
                 if constexpr (V == 4) {
-                    const float4 x = __ldg(reinterpret_cast<const float4*>(X + p * D + j));
+                    const float4 x = __ldg(reinterpret_cast<const float4*>(X + src * D + j));
                     const float4 m = __ldg(reinterpret_cast<const float4*>(mu + j));
                     v[0] = x.x - m.x; v[1] = x.y - m.y; v[2] = x.z - m.z; v[3] = x.w - m.w;
                 } else {
-                    v[0] = X[p * D + j] - __ldg(mu + j);
+                    v[0] = X[src * D + j] - __ldg(mu + j);
                 }
             }
             if (to_bf16) {
@@ -277,7 +275,7 @@ prep_rows_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
             norms[p] = (p < N) ? nf : __int_as_float(0x7f800000);
             rho[p] = rf;
             const float n32 = __fadd_rn(vh, vl);   // ||v||^2 of the float32 operand v
-            if (norms32) norms32[p] = (p < N) ? n32 : __int_as_float(0x7f800000);
+            if (norms32) norms32[src] = (p < N) ? n32 : __int_as_float(0x7f800000);
             if (p < N) {
                 my_n = max(my_n, __float_as_uint(nf));
                 my_r = max(my_r, __float_as_uint(rf));
@@ -330,6 +328,7 @@ prep_rows_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
 // leaves open (nothing runs when *open_count is 0): with v = fl(x - mu) and
 // h = bf16(v) (the candidate operand xt), the second term l = bf16(v - h)
 // (v - h is exact), so that s = h + l carries 16 significant bits of v:
+//   xh[p]      = h (nullable: only where the operand xt is in another order),
 //   xl[p]      = l,
 //   norms_s[p] = ||s||^2 (s = h + l is exact in float32: l either equals
 //                v - h, then s = v, or has its last bit above v's),
@@ -341,8 +340,8 @@ template <int V>
 __global__ void __launch_bounds__(256)
 prep_split_kernel(const float* __restrict__ X, int64_t N, int D, int Dp, int64_t Np,
                   const float* __restrict__ mu, const long long* __restrict__ open_count,
-                  __nv_bfloat16* __restrict__ xl, float* __restrict__ norms_s,
-                  float* __restrict__ rho_s, DevState* st) {
+                  __nv_bfloat16* __restrict__ xh, __nv_bfloat16* __restrict__ xl,
+                  float* __restrict__ norms_s, float* __restrict__ rho_s, DevState* st) {
     if (*open_count == 0) return;
     __shared__ unsigned bmax_n, bmax_r, bmax_k;
     if (threadIdx.x == 0) { bmax_n = 0u; bmax_r = 0u; bmax_k = 0u; }
@@ -371,11 +370,12 @@ prep_split_kernel(const float* __restrict__ X, int64_t N, int D, int Dp, int64_t
                     v[0] = X[p * D + j] - __ldg(mu + j);
                 }
             }
-            __nv_bfloat16 lb[V];
+            __nv_bfloat16 hb[V], lb[V];
             float sv[V];
 #pragma unroll
             for (int q = 0; q < V; ++q) {
-                const float h = __bfloat162float(__float2bfloat16_rn(v[q]));
+                hb[q] = __float2bfloat16_rn(v[q]);
+                const float h = __bfloat162float(hb[q]);
                 lb[q] = __float2bfloat16_rn(v[q] - h);
                 sv[q] = h + __bfloat162float(lb[q]);
             }
@@ -386,8 +386,15 @@ prep_split_kernel(const float* __restrict__ X, int64_t N, int D, int Dp, int64_t
                 w.x = *reinterpret_cast<const unsigned*>(&b01);
                 w.y = *reinterpret_cast<const unsigned*>(&b23);
                 *reinterpret_cast<uint2*>(xl + p * Dp + j) = w;
+                if (xh) {
+                    b01.x = hb[0]; b01.y = hb[1]; b23.x = hb[2]; b23.y = hb[3];
+                    w.x = *reinterpret_cast<const unsigned*>(&b01);
+                    w.y = *reinterpret_cast<const unsigned*>(&b23);
+                    *reinterpret_cast<uint2*>(xh + p * Dp + j) = w;
+                }
             } else {
                 xl[p * Dp + j] = lb[0];
+                if (xh) xh[p * Dp + j] = hb[0];
             }
 #pragma unroll
             for (int q = 0; q < V; ++q) {
@@ -836,11 +843,10 @@ __device__ __forceinline__ float exact_d2(const float* __restrict__ xp,
 #endif
 constexpr int kRerankUnroll = SLK_RERANK_UNROLL;
 
-// Rerank + certificate, one warp per row.  Lists hold KC entries each; the
-// SEL best of their union (SEL >= KC: several lists of a split together, as
-// the two column halves of the 8-warp tensor-core kernel) are the candidates
-// whose last one bounds the rest.  gam bounds the error of a tile's dot
-// product relative to |xt_p| |xt_q| (with the norms' roundings added here).
+// Rerank + certificate of the float32 tiles, one warp per row.  Lists hold KC
+// entries each; the KC best of their union are the candidates whose last one
+// bounds the rest.  gam bounds the error of a tile's dot product relative to
+// |xt_p| |xt_q| (with the norms' roundings added here).
 //   MODE 0: every row p < N, the lists of the candidate kernels at
 //           ((list Np + p) KC), failures appended to fb_list.
 //   MODE 1: the rows fb_in[f], f < F = *count_in, their float32 query lists
@@ -848,11 +854,7 @@ constexpr int kRerankUnroll = SLK_RERANK_UNROLL;
 //           list buffer's capacity in floats), norms of the float32 operand
 //           (rho <= u ||v||), failures appended to fb_list / *count_out; for
 //           F <= kExactDirectRows every row is appended (no lists were made).
-//   MODE 2: the rows fb_in[f], f < *count_in, their two-term bfloat16 query
-//           lists at ((list Np + f) KC) for f < Np (Np: the query stage's
-//           row capacity), norms and rho of the two-term operand; the rows
-//           from Np on, and the failures, appended to fb_list / *count_out.
-template <int KC, int MODE, int E = MAXE, int SEL = KC>
+template <int KC, int MODE, int E = MAXE>
 __global__ void __launch_bounds__(256, 4)
 knn_rerank_kernel(const float* __restrict__ X, int64_t N, int D, int Dp, int k, int splits_in,
                   int64_t Np, const float* __restrict__ cand_d, const int32_t* __restrict__ cand_i,
@@ -862,6 +864,7 @@ knn_rerank_kernel(const float* __restrict__ X, int64_t N, int D, int Dp, int k, 
                   const int32_t* __restrict__ fb_in = nullptr, const long long* count_in = nullptr,
                   long long* count_out = nullptr) {
     constexpr bool Q = MODE != 0;
+    constexpr int SEL = KC;
     __shared__ float s_d[8][32 * E];   // each warp's staged lists (256 threads)
     __shared__ int s_i[8][32 * E];
     __shared__ float s_od[8][SEL];     // and its SEL selected candidates
@@ -869,15 +872,12 @@ knn_rerank_kernel(const float* __restrict__ X, int64_t N, int D, int Dp, int k, 
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
     const double u = 5.9604644775390625e-08;  // 2^-24
-    const double nmax = (double)__uint_as_float(
-        MODE == 0 ? st->knn_max_norm_bits : MODE == 1 ? st->knn_max_norm32_bits : st->knn_max_norm_s_bits);
+    const double nmax = (double)__uint_as_float(MODE == 0 ? st->knn_max_norm_bits : st->knn_max_norm32_bits);
     const double rmax = MODE == 1 ? u * sqrt(nmax) * (1.0 + 1e-6)
-                                  : (double)__uint_as_float(MODE == 0 ? st->knn_max_rho_bits
-                                                                      : st->knn_max_rho_s_bits);
+                                  : (double)__uint_as_float(st->knn_max_rho_bits);
     // rho_q <= kappa ||v_q|| for every row q
     const double kappa = MODE == 1 ? u * (1.0 + 1e-5)
-                                   : (double)__uint_as_float(MODE == 0 ? st->knn_max_kappa_bits
-                                                                       : st->knn_max_kappa_s_bits);
+                                   : (double)__uint_as_float(st->knn_max_kappa_bits);
     const double err_exact = 1.01 * (double)(D + 8) * u;
     // float32 copies of the bound's constants for the candidate pruning
     // (margins of 1e-6 .. 1e-5 cover the float rounding of the bounds)
@@ -901,14 +901,6 @@ knn_rerank_kernel(const float* __restrict__ X, int64_t N, int D, int Dp, int k, 
     for (int64_t f = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); f < rows;
          f += nw) {
         const int64_t p = Q ? (int64_t)fb_in[f] : f;
-        if (MODE == 2 && f >= Np) {
-            // beyond the query stage's capacity: on to the next stage
-            if (lane == 0) {
-                const unsigned long long slot = atomicAdd((unsigned long long*)count_out, 1ull);
-                fb_list[slot] = (int32_t)p;
-            }
-            continue;
-        }
         if (!Q && lane == 0) row_ptr[p] = p * (int64_t)k;
         // The splits' lists are sorted by (distance, index) and cover
         // disjoint columns, so the position of an entry in their union is its
@@ -1173,6 +1165,273 @@ knn_rerank_kernel(const float* __restrict__ X, int64_t N, int D, int Dp, int k, 
                 fb_list[slot] = (int32_t)p;
             }
         }
+    }
+}
+
+// ------------------------------------------- selection from the sweep's lists
+
+// The warp's need mask m over candidates (lane b holds candidate b, its point
+// in q_of): exact distances, lane b receives that of candidate b.
+__device__ __forceinline__ void exact_of(const float* __restrict__ X, const float* __restrict__ xp, int D,
+                                         int lane, unsigned m, int q_of, float& mine) {
+    if (D > 256) {
+        // long rows: a candidate's own loads already overlap
+        for (; m != 0u; m &= m - 1u) {
+            const int b = __ffs(m) - 1;
+            const int q = __shfl_sync(0xffffffffu, q_of, b);
+            const float d = exact_d2(xp, X + (int64_t)q * D, D, lane);
+            if (lane == b) mine = d;
+        }
+        return;
+    }
+    // short rows: four candidates at a time, their row gathers overlap; each
+    // one's sum has exact_d2's per-lane order and butterfly (the same bits)
+    while (m != 0u) {
+        int b[4], q[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            b[c] = m != 0u ? __ffs(m) - 1 : -1;
+            if (m != 0u) m &= m - 1u;
+            q[c] = __shfl_sync(0xffffffffu, q_of, b[c] < 0 ? 0 : b[c]);
+        }
+        float part[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll kRerankUnroll
+        for (int j = lane; j < D; j += 32) {
+            const float a = xp[j];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (b[c] >= 0) {
+                    const float df = a - X[(int64_t)q[c] * D + j];
+                    part[c] = fmaf(df, df, part[c]);
+                }
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) part[c] += __shfl_xor_sync(0xffffffffu, part[c], o);
+            if (b[c] >= 0 && lane == b[c]) mine = part[c];
+        }
+    }
+}
+
+struct SelectArgs {
+    const float* X;
+    int64_t N;
+    int D, Dp, k;
+    SweepWork w;
+    SweepLists lists;
+    const int32_t* perm;      // point of each operand column (NULL: the same)
+    const float* norms;       // by operand column
+    const float* rho;
+    double gam;
+    int64_t* row_ptr;
+    int32_t* col_idx;
+    float* dist2;
+    int32_t* fb_list;         // rows left open, counted in *fb_count
+    unsigned long long* fb_count;
+    const DevState* st;
+    // two-term stage: rows fb_in[f], f < *count_in; those from cap on are left open
+    const int32_t* fb_in;
+    const long long* count_in;
+    int64_t cap;
+};
+
+// k-th smallest dt of a row over the lists of its pieces.  A piece's list holds
+// the columns under its own threshold, its k smallest among them, so the
+// entries up to the smallest k-th value of any piece (at most k per piece)
+// contain the k smallest of the union; ranks by counting.
+template <int NK>
+__device__ __forceinline__ float union_kth(const SweepLists& ls, int64_t first, int segs,
+                                           int64_t extra0, int fr, float kmin, int k, float* sk, int lane,
+                                           bool& bad) {
+    int m = 0;
+    for (int s = 0; s < segs; ++s) {
+        const int64_t row = s == 0 ? first : (extra0 + s) * 128 + fr;
+        const uint2* src = ls.cand + row * ls.stride;
+        const int n = sweep_count(src[0].x);
+        for (int e0 = 0; e0 < n; e0 += 32) {
+            const float d = e0 + lane < n ? __uint_as_float(src[1 + e0 + lane].x) : kInf;
+            const unsigned take = __ballot_sync(0xffffffffu, d <= kmin && d < kInf);
+            const int at = m + __popc(take & ((1u << lane) - 1u));
+            if (d <= kmin && d < kInf && at < NK) sk[at] = d;
+            m += __popc(take);
+        }
+    }
+    if (m > NK || m < k) { bad = true; return kInf; }
+    __syncwarp();
+    float found = -kInf;
+    for (int e = lane; e < m; e += 32) {
+        const float d = sk[e];
+        int less = 0, leq = 0;
+        for (int c = 0; c < m; ++c) {
+            less += sk[c] < d;
+            leq += sk[c] <= d;
+        }
+        if (less < k && k <= leq) found = d;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) found = fmaxf(found, __shfl_xor_sync(0xffffffffu, found, o));
+    __syncwarp();
+    return found;
+}
+
+// The k nearest of each row from the candidates the sweep kept, one warp per
+// row: the threshold of the k-th smallest dt over all pieces, exact float32
+// distances of the candidates whose lower bound can still reach the k nearest,
+// the k smallest by (distance, index).  Every column that is no candidate has
+// dt >= T (or a squared operand distance >= T), which certifies the row unless
+// its k-th exact distance is too close to that (knn_cert.cuh); it is also left
+// open if a list gave up on ties or more than 64 candidates remain (128 in the
+// two-term stage, whose row blocks come in more pieces).
+template <bool SPLIT>
+__global__ void __launch_bounds__(256, 4)
+knn_select_kernel(const SelectArgs a) {
+    constexpr int NK = kSweepMaxSeg * SLK_MAX_K;
+    __shared__ float s_k[8][NK];
+    constexpr int kSelMax = SPLIT ? 128 : 64, CPL = kSelMax / 32;
+    __shared__ float s_d[8][kSelMax];
+    __shared__ int s_i[8][kSelMax];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, k = a.k, D = a.D;
+    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const DevState* st = a.st;
+    const CertConsts cc = SPLIT ? cert_make(a.gam, a.Dp, D, st->knn_max_norm_s_bits, st->knn_max_rho_s_bits,
+                                            st->knn_max_kappa_s_bits)
+                                : cert_make(a.gam, a.Dp, D, st->knn_max_norm_bits, st->knn_max_rho_bits,
+                                            st->knn_max_kappa_bits);
+    SweepWork w = a.w;
+    int64_t rows = a.N;
+    if (SPLIT) {
+        rows = (int64_t)(*(const volatile long long*)a.count_in);
+        const int64_t in = rows < a.cap ? rows : a.cap;
+        w.row_blocks = (int)((in + 127) / 128);
+    }
+    const int64_t chunk = sweep_chunk(w, sweep_total(w));
+    if (!SPLIT && blockIdx.x == 0 && threadIdx.x == 0) a.row_ptr[a.N] = a.N * (int64_t)k;
+    for (int64_t f = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib; f < rows; f += nw) {
+        const int64_t c0 = SPLIT ? (int64_t)a.fb_in[f] : f;   // the row's own operand column
+        const int64_t p = a.perm ? (int64_t)a.perm[c0] : c0;
+        bool bad = SPLIT && f >= a.cap;   // beyond the query stage's capacity: on to the next stage
+        int nc = 0;
+        float T = kInf, lim = kInf;   // columns that are no candidate have dt >= T
+        const float np_ = a.norms[c0];
+        const float sp = sqrtf(np_) * cc.sn_infl, rp = a.rho[c0] * 1.000001f;
+        if (!SPLIT && lane == 0) a.row_ptr[p] = p * (int64_t)k;
+        if (!bad) {
+            const int rb = (int)(f >> 7), fr = (int)(f & 127);
+            int64_t s0, s1;
+            sweep_block(w, rb, s0, s1);
+            const int64_t u0 = s0 / chunk;
+            const int segs = s1 > s0 ? (int)((s1 - 1) / chunk - u0) + 1 : 1;
+            const int64_t extra0 = (int64_t)a.w.row_blocks + u0;   // slot of piece s > 0: extra0 + s
+            // headers of the pieces
+            int n = 0;
+            float kt = kInf, tc = kInf;
+            if (lane < segs) {
+                const int64_t row = lane == 0 ? f : (extra0 + lane) * 128 + fr;
+                const uint2* src = a.lists.cand + row * a.lists.stride;
+                const uint2 h = src[0];
+                n = sweep_count(h.x);
+                kt = __uint_as_float(h.y);
+                if (sweep_capped(h.x)) tc = __uint_as_float(src[1 + n].x);
+            }
+            bad = __any_sync(0xffffffffu, n < 0);
+            float dk = kt;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                dk = fminf(dk, __shfl_xor_sync(0xffffffffu, dk, o));
+                tc = fminf(tc, __shfl_xor_sync(0xffffffffu, tc, o));
+            }
+            if (!bad && segs > 1)
+                dk = union_kth<NK>(a.lists, f, segs, extra0, fr, dk, k, s_k[wib], lane, bad);
+            if (!(dk < kInf)) bad = true;
+            if (!bad) {
+                T = fminf(tc, cert_thr(cc, sp, rp, dk));
+                const float sk = cert_reach(cc, sp, rp, dk);
+                lim = sk * sk * 1.00001f + 1e-30f;
+                for (int s = 0; s < segs; ++s) {
+                    const int64_t row = s == 0 ? f : (extra0 + s) * 128 + fr;
+                    const uint2* src = a.lists.cand + row * a.lists.stride;
+                    const int ns = __shfl_sync(0xffffffffu, n, s);
+                    for (int e0 = 0; e0 < ns; e0 += 32) {
+                        const bool in = e0 + lane < ns;
+                        const uint2 v = in ? src[1 + e0 + lane] : make_uint2(0u, 0u);
+                        const bool take = in && __uint_as_float(v.x) < T;
+                        const unsigned tm = __ballot_sync(0xffffffffu, take);
+                        const int at = nc + __popc(tm & ((1u << lane) - 1u));
+                        if (take && at < kSelMax) {
+                            s_d[wib][at] = __uint_as_float(v.x);
+                            s_i[wib][at] = (int)v.y;
+                        }
+                        nc += __popc(tm);
+                    }
+                }
+                if (nc > kSelMax || nc < k) bad = true;
+            }
+        }
+        if (bad) {
+            if (lane == 0) a.fb_list[atomicAdd(a.fb_count, 1ull)] = (int32_t)p;
+            continue;
+        }
+        __syncwarp();
+        // candidate c lives on lane c % 32, slot c / 32; one whose lower bound
+        // (its own norm and rho) exceeds the reach of the k nearest needs no
+        // exact distance
+        int ci[CPL];
+        float myd[CPL];
+        unsigned need[CPL];
+#pragma unroll
+        for (int h = 0; h < CPL; ++h) {
+            const int c = lane + 32 * h;
+            bool keep = false;
+            ci[h] = kNoIdx;
+            myd[h] = kInf;
+            need[h] = 0u;
+            if (32 * h >= nc) continue;   // warp-uniform
+            if (c < nc) {
+                const int q = s_i[wib][c];
+                ci[h] = a.perm ? a.perm[q] : q;
+                const float rq = a.rho[q] * 1.000001f;
+                const float snq = sp + sqrtf(a.norms[q]) * cc.sn_infl;
+                const float lo = s_d[wib][c] - cc.coef * snq * snq;
+                const float r = lo > 0.f ? sqrtf(lo) * 0.99999f - (rp + rq) : 0.f;
+                const float lb = r > 0.f ? r * r * 0.99999f : 0.f;
+                keep = !(lb > lim);
+            }
+            need[h] = __ballot_sync(0xffffffffu, keep);
+        }
+        __syncwarp();
+        const float* xp = a.X + p * D;
+#pragma unroll
+        for (int h = 0; h < CPL; ++h) exact_of(a.X, xp, D, lane, need[h], ci[h], myd[h]);
+        // rank of each candidate by (exact distance, index) among the computed
+        // ones; a skipped one (+inf) ranks after at least k of them
+        int rank[CPL];
+#pragma unroll
+        for (int h = 0; h < CPL; ++h) rank[h] = 0;
+#pragma unroll
+        for (int hs = 0; hs < CPL; ++hs) {
+            for (unsigned m = need[hs]; m != 0u; m &= m - 1u) {
+                const int b = __ffs(m) - 1;
+                const float od = __shfl_sync(0xffffffffu, myd[hs], b);
+                const int oi = __shfl_sync(0xffffffffu, ci[hs], b);
+#pragma unroll
+                for (int h = 0; h < CPL; ++h)
+                    if (lex_less(od, oi, myd[h], ci[h])) ++rank[h];
+            }
+        }
+        float dk = kInf;
+#pragma unroll
+        for (int h = 0; h < CPL; ++h) {
+            if (lane + 32 * h < nc && rank[h] < k) {
+                a.col_idx[p * k + rank[h]] = ci[h];
+                a.dist2[p * k + rank[h]] = myd[h];
+                if (rank[h] == k - 1) dk = myd[h];
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dk = fminf(dk, __shfl_xor_sync(0xffffffffu, dk, o));
+        if (lane == 0 && !cert_ok(cc, sp, rp, dk, T)) a.fb_list[atomicAdd(a.fb_count, 1ull)] = (int32_t)p;
     }
 }
 
@@ -1506,16 +1765,31 @@ int choose_kc(int k) { return (k + 4 <= 16) ? 16 : 32; }
 struct KnnPlan {
     int64_t Np;
     int Dp, kc, splits, row_blocks, n_tiles;
-    int ew;      // epilogue warps of the tensor-core kernel (lists per split: ew / 4)
-    int lists;   // candidate lists per row: splits x lists per split
     bool bf16;
     bool aug;    // tensor-core tiles with the norms folded into one more K slice
+    // tensor-core sweep: CTAs, entries of a row list, and whether its work is
+    // cut only between row blocks (no lists beyond one per row)
+    int units, stride, aligned;
     // two-term stage (bfloat16 and N >= kTwoTermMinRows): row capacity (a
-    // multiple of 128), column splits and lists (of 32) per row
+    // multiple of 128) and CTAs
     bool two_term;
     int64_t fcap;
-    int ssplits, slists;
+    int sunits;
+    // points sorted by region, tiles out of reach left out (knn_group.cu)
+    bool grouped;
 };
+
+// Sweeps shorter than this are not worth the sort's launches (0.15 to 0.2 ms).
+// Tiles per CTA times K slices and their fixed part: 490 at 19937 x 256 (0.46 ms
+// grouped, 0.47 not), 1060 at 30000 x 64 (0.43 and 0.77), 14800 at 70000 x 784
+// with 10 clusters (1.66 and 5.77; with one cluster, where nothing can be left
+// out, 6.52 and 5.81).
+constexpr int64_t kGroupMinWork = 500;
+// Tiles around a row block's own columns that the first pass takes: 4, and 8
+// from 2000 column tiles on, where regions are longer (4 against 8: 0.39 and
+// 0.45 ms at 42099 x 64, 4.93 and 5.23 at 200000 x 128, 88.7 and 85.5 at 1e6 x
+// 128).
+int group_window(int n_tiles) { return n_tiles < 2000 ? 4 : 8; }
 
 // Rows the two-term tensor-core stage takes at most (fewer at large D, see
 // make_plan); the open rows beyond it go to the float32 stage.
@@ -1524,52 +1798,50 @@ constexpr int64_t kSplitRowCap = 65536;
 // tiles over N points are cheap there, and the two-term stage's four launches
 // would cost more than they save: the batched form runs many such graphs).
 constexpr int64_t kTwoTermMinRows = 100000;
+constexpr int kTcCols = 256;   // columns of a tensor-core tile
 
-// Column splits for the persistent tensor-core kernel.  Every split restarts
-// the rows' candidate lists, so prefer few, long work items (row block x
-// split) of at least 8 column tiles: the smallest split count whose last
-// round is at least 95 % full, else the best-filled one.
-int tc_splits(int row_blocks, int n_tiles, int num_sms, int max_splits) {
-    int best = 1;
-    double best_eff = -1.0;
-    const int s_max = std::max(1, std::min(max_splits, n_tiles / 8));
-    for (int s = 1; s <= s_max; ++s) {
-        const int64_t items = (int64_t)row_blocks * s;
-        const int64_t rounds = (items + num_sms - 1) / num_sms;
-        const double eff = (double)items / (double)(rounds * num_sms);
-        if (eff >= 0.95) return s;
-        if (eff > best_eff + 1e-9) { best_eff = eff; best = s; }
-    }
-    return best;
-}
+size_t plan_bytes(const KnnPlan& pl, int64_t N, int D);
 
-KnnPlan make_plan(const slk_ctx* ctx, int64_t N, int D, int k, int precision) {
+// The plan, within `budget` bytes of workspace: with too little for row lists
+// of 64 entries and one list more per CTA, lists of 32 and whole row blocks
+// per CTA (slower, more rows left open; the same graph).
+KnnPlan make_plan(const slk_ctx* ctx, int64_t N, int D, int k, int precision, size_t budget) {
     KnnPlan pl{};
     pl.bf16 = (precision == SLK_KNN_BF16_RERANK);
-    // bfloat16 candidates carry a larger rounding error: keep about 5k
-    // candidates per row and split so that the certificate still holds for
-    // most rows -- for k > 6 two lists of 32 (the column halves of every
-    // tile, one per epilogue warp of a pair), whose smaller last entry
-    // bounds every rejected column like the last entry of one list of 64
-#ifndef SLK_TC_BF16_KC64
-#define SLK_TC_BF16_KC64 0
-#endif
-    pl.kc = pl.bf16 ? ((k <= 6 || !SLK_TC_BF16_KC64) ? 32 : 64) : choose_kc(k);
-    pl.ew = (pl.bf16 && k > 6 && pl.kc == 32) ? 8 : 4;
-    // where the tiles' epilogue outweighs their MMAs (small D), fold the
-    // norms into the MMAs: the epilogue then reads no norms and takes no
-    // barrier per tile
-#ifndef SLK_TC_AUG_MAX_DP
-#define SLK_TC_AUG_MAX_DP 256
-#endif
+    pl.kc = choose_kc(k);
     // the tensor-core tiles read 256-row column tiles: keep them inside the matrix
     pl.Np = (int64_t)align_up((size_t)N, pl.bf16 ? 256 : 128);
     pl.Dp = (int)align_up((size_t)D, pl.bf16 ? 64 : BK);
-    pl.aug = pl.bf16 && pl.kc == 32 && pl.Dp <= SLK_TC_AUG_MAX_DP;
     pl.row_blocks = (int)(pl.Np / BM);
+    const int sms = ctx->num_sms > 0 ? ctx->num_sms : 148;
+    if (pl.bf16) {
+        // where the tiles' epilogue outweighs their MMAs (small D), fold the
+        // norms into the MMAs: the epilogue then reads no norms
+        pl.aug = pl.Dp <= 256;
+        pl.n_tiles = (int)(pl.Np / kTcCols);
+        const int64_t tiles = (int64_t)pl.row_blocks * pl.n_tiles;
+        pl.units = (int)std::min<int64_t>(sms, tiles);
+        // two-term query rows: at most 65536, and operands (h and l) of at most 64 MiB
+        const int64_t by_mem = std::max<int64_t>(128, ((int64_t)1 << 24) / pl.Dp / 128 * 128);
+        pl.fcap = std::min<int64_t>(std::min<int64_t>((int64_t)align_up((size_t)N, 128), kSplitRowCap),
+                                    by_mem);
+        pl.sunits = (int)std::min<int64_t>(sms, 4 * (pl.fcap / 128));
+        pl.two_term = N >= kTwoTermMinRows;
+        pl.stride = kSweepStride;
+        pl.aligned = 0;
+        // the tile table must stay a small part of the workspace
+        pl.grouped = tiles / pl.units * (2 + pl.Dp / 64) >= kGroupMinWork && pl.n_tiles < 65536 &&
+                     pl.n_tiles > 16 && pl.n_tiles <= 32 * (kSweepStride * 8 + 2 * pl.Dp);
+        if (pl.grouped && plan_bytes(pl, N, D) > budget) pl.grouped = false;
+        if (plan_bytes(pl, N, D) > budget) {
+            pl.stride = 32;
+            pl.aligned = 1;
+        }
+        return pl;
+    }
     pl.n_tiles = (int)(pl.Np / BN);
     const int max_splits = (32 * MAXE) / pl.kc;
-    const int cap = 2 * (ctx->num_sms > 0 ? ctx->num_sms : 148);  // resident CTAs
+    const int cap = 2 * sms;  // resident CTAs
     // smallest split count giving >= 2 waves, then the one with the best wave fill
     int best = 1;
     double best_eff = -1.0;
@@ -1582,53 +1854,74 @@ KnnPlan make_plan(const slk_ctx* ctx, int64_t N, int D, int k, int precision) {
         if (total >= 8 * cap) break;
     }
     pl.splits = best;
-    pl.lists = pl.splits;
-    if (pl.bf16) {
-        const int per = knn_tc_lists_per_split(pl.kc, pl.ew);
-        const int tiles_tc = (int)((pl.Np + knn_tc_tile_cols() - 1) / knn_tc_tile_cols());
-        pl.splits = tc_splits(pl.row_blocks, tiles_tc, ctx->num_sms > 0 ? ctx->num_sms : 148,
-                              max_splits / per);
-        pl.lists = pl.splits * per;
-        // the open rows are few: split the columns as far as the rerank's
-        // staging (32 MAXE entries per row) and 8 tiles per item allow
-        // at most 65536 rows, and query operands (h and l) of at most 64 MiB
-        const int64_t by_mem = std::max<int64_t>(128, ((int64_t)1 << 24) / pl.Dp / 128 * 128);
-        pl.fcap = std::min<int64_t>(std::min<int64_t>((int64_t)align_up((size_t)N, 128), kSplitRowCap),
-                                    by_mem);
-        pl.ssplits = std::max(1, std::min((32 * MAXE) / (32 * per), tiles_tc / 8));
-        pl.slists = pl.ssplits * per;
-        pl.two_term = N >= kTwoTermMinRows;
-    }
     return pl;
+}
+
+// Row lists of the sweeps (rows of 128-row slots).
+size_t sweep_rows(const KnnPlan& pl) {
+    return (size_t)pl.Np + (pl.aligned ? 0 : (size_t)pl.units * 128);
+}
+// Floats of one of the two halves of the candidate buffer (distances, indices).
+size_t cand_floats(const KnnPlan& pl) {
+    return pl.bf16 ? sweep_rows(pl) * pl.stride : (size_t)pl.splits * pl.Np * pl.kc;
+}
+
+// The scratch of a graph, in the order of knn_graph_launch.
+struct KnnBufs {
+    double* colsum;
+    void* xt;
+    float *norms, *rho, *cand_d;
+    int32_t *cand_i, *fb;
+    float *norms32, *mu;
+    int32_t* fb2;
+    __nv_bfloat16* xl16;
+    float *norms_s, *rho_s;
+    __nv_bfloat16 *qh, *ql;
+    float* qnorm;
+    uint2* scand;
+    __nv_bfloat16* aug;
+    GroupBufs grp;
+};
+KnnBufs carve_knn(WsCarver& wc, const KnnPlan& pl, int64_t N, int D) {
+    KnnBufs b{};
+    b.colsum = wc.take<double>(D);
+    b.xt = wc.take<unsigned char>((pl.bf16 ? 2 : 4) * (size_t)pl.Np * pl.Dp);
+    b.norms = wc.take<float>(pl.Np);
+    b.rho = wc.take<float>(pl.Np);
+    // one block: float32 lists in two halves, the sweep's lists as pairs
+    b.cand_d = wc.take<float>(2 * cand_floats(pl));
+    b.cand_i = reinterpret_cast<int32_t*>(b.cand_d + cand_floats(pl));
+    b.fb = wc.take<int32_t>(N);
+    b.norms32 = wc.take<float>(pl.Np);
+    b.mu = wc.take<float>(D);
+    b.fb2 = wc.take<int32_t>(N);
+    if (pl.bf16 && pl.two_term) {
+        b.xl16 = wc.take<__nv_bfloat16>((size_t)pl.Np * pl.Dp);
+        b.norms_s = wc.take<float>(pl.Np);
+        b.rho_s = wc.take<float>(pl.Np);
+        b.qh = wc.take<__nv_bfloat16>((size_t)pl.fcap * pl.Dp);
+        b.ql = wc.take<__nv_bfloat16>((size_t)pl.fcap * pl.Dp);
+        b.qnorm = wc.take<float>(pl.fcap);
+        b.scand = wc.take<uint2>(((size_t)pl.fcap + (size_t)pl.sunits * 128) * kSweepStride);
+    }
+    if (pl.aug) b.aug = wc.take<__nv_bfloat16>(32 * (size_t)pl.Np);
+    if (pl.grouped) group_carve(wc, b.grp, N, pl.Np, pl.Dp, pl.n_tiles);
+    return b;
+}
+size_t plan_bytes(const KnnPlan& pl, int64_t N, int D) {
+    WsCarver wc(nullptr);
+    carve_knn(wc, pl, N, D);
+    return wc.off + 4096;
 }
 
 }  // namespace
 
 size_t knn_ws_bytes(const slk_ctx* ctx, int64_t N, int D, int k, int precision) {
-    const KnnPlan pl = make_plan(ctx, N, D, k, precision);
-    size_t b = 0;
-    b += align_up(sizeof(double) * D, 256);
-    b += align_up((pl.bf16 ? 2 : 4) * (size_t)pl.Np * pl.Dp, 256);
-    b += 2 * align_up(sizeof(float) * pl.Np, 256);
-    b += 2 * align_up(sizeof(float) * (size_t)pl.lists * pl.Np * pl.kc, 256);
-    b += align_up(sizeof(float) * pl.Np, 256) + align_up(sizeof(float) * D, 256);   // norms32, mu
-    b += align_up(sizeof(int32_t) * N, 256);                                         // second list
-    b += align_up(sizeof(int32_t) * (size_t)N, 256);
-    if (pl.aug) b += align_up(2 * 32 * (size_t)pl.Np, 256);   // folded-norm columns
-    if (pl.bf16 && pl.two_term) {
-        // two-term stage: xl, norms_s, rho_s, query rows (h, l, norms), lists
-        b += align_up(2 * (size_t)pl.Np * pl.Dp, 256) + 2 * align_up(sizeof(float) * pl.Np, 256);
-        b += 2 * align_up(2 * (size_t)pl.fcap * pl.Dp, 256) + align_up(sizeof(float) * pl.fcap, 256);
-        b += 2 * align_up(sizeof(float) * (size_t)pl.slists * pl.fcap * 32, 256);
-    }
-    if (pl.bf16) b += align_up(sizeof(int32_t) * (size_t)N, 256);   // third list
-    return b + 4096;
+    return plan_bytes(make_plan(ctx, N, D, k, precision, SIZE_MAX), N, D);
 }
-
-slk_status knn_cand_bf16_launch(slk_ctx* ctx, const __nv_bfloat16* xt, const float* norms,
-                                const __nv_bfloat16* aug, int64_t N, int Dp, int64_t Np, int kc,
-                                int ew, int splits, float* cand_d, int32_t* cand_i,
-                                unsigned int* err_flag, unsigned long long* sweep);
+size_t knn_ws_min_bytes(const slk_ctx* ctx, int64_t N, int D, int k, int precision) {
+    return plan_bytes(make_plan(ctx, N, D, k, precision, 0), N, D);
+}
 
 namespace {
 
@@ -1636,7 +1929,8 @@ namespace {
 // loads where the row layout and the summation bound allow them.
 slk_status launch_prep(slk_ctx* ctx, const float* X, int64_t N, int D, int Dp, int64_t Np,
                        double* colsum, float* mu, float* xt32, __nv_bfloat16* xt16,
-                       float* norms, float* rho, float* norms32, __nv_bfloat16* aug, DevState* st) {
+                       float* norms, float* rho, float* norms32, __nv_bfloat16* aug, const GroupBufs* grp,
+                       DevState* st) {
     cudaStream_t s = ctx->stream;
     const bool v4 = D % 4 == 0 && Dp >= 128 && (reinterpret_cast<uintptr_t>(X) & 15) == 0 &&
                     (reinterpret_cast<uintptr_t>(mu) & 15) == 0;
@@ -1649,15 +1943,21 @@ slk_status launch_prep(slk_ctx* ctx, const float* X, int64_t N, int D, int Dp, i
     else col_sum_kernel<1><<<cgrid, dim3(32, 8), 0, s>>>(X, N, D, colsum);
     mu_kernel<<<(D + 255) / 256, 256, 0, s>>>(colsum, N, D, mu);
     SLK_LAUNCH_CHECK(ctx, "col_sum_kernel");
+    const int32_t* perm = nullptr;
+    if (grp) {
+        const slk_status r = group_order_launch(ctx, *grp, X, N, D, Dp, mu);
+        if (r != SLK_OK) return r;
+        perm = grp->perm;
+    }
     int64_t pg = (Np + 7) / 8;
     if (pg > (int64_t)ctx->num_sms * 64) pg = (int64_t)ctx->num_sms * 64;
     const int to_bf16 = xt16 != nullptr ? 1 : 0;
     if (v4)
         prep_rows_kernel<4><<<(unsigned)pg, 256, 0, s>>>(X, N, D, Dp, Np, mu, to_bf16, xt32, xt16,
-                                                         norms, rho, norms32, aug, st);
+                                                         norms, rho, norms32, aug, perm, st);
     else
         prep_rows_kernel<1><<<(unsigned)pg, 256, 0, s>>>(X, N, D, Dp, Np, mu, to_bf16, xt32, xt16,
-                                                         norms, rho, norms32, aug, st);
+                                                         norms, rho, norms32, aug, perm, st);
     SLK_LAUNCH_CHECK(ctx, "prep_rows_kernel");
     return SLK_OK;
 }
@@ -1671,40 +1971,23 @@ slk_status knn_prep_fp32_launch(slk_ctx* ctx, const float* X, int64_t N, int D, 
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(colsum, 0, sizeof(double) * D, s));
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(&st->knn_max_norm_bits, 0, 2 * sizeof(unsigned int), s));
     SLK_COUNT_LAUNCH(ctx, 2);
-    return launch_prep(ctx, X, N, D, Dp, Np, colsum, mu, xt, nullptr, norms, rho, nullptr, nullptr, st);
+    return launch_prep(ctx, X, N, D, Dp, Np, colsum, mu, xt, nullptr, norms, rho, nullptr, nullptr,
+                       nullptr, st);
 }
 
 slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int k,
                             int precision, int64_t* row_ptr, int32_t* col_idx, float* dist2,
-                            void* ws, DevState* st) {
-    const KnnPlan pl = make_plan(ctx, N, D, k, precision);
+                            void* ws, size_t ws_bytes, DevState* st) {
+    const KnnPlan pl = make_plan(ctx, N, D, k, precision, ws_bytes);
     ctx->knn_last_bf16 = pl.bf16;
     ctx->knn_last_two_term = pl.bf16 && pl.two_term;
     WsCarver wc(ws);
-    double* colsum = wc.take<double>(D);
-    void* xt = wc.take<unsigned char>((pl.bf16 ? 2 : 4) * (size_t)pl.Np * pl.Dp);
-    float* norms = wc.take<float>(pl.Np);
-    float* rho = wc.take<float>(pl.Np);
-    float* cand_d = wc.take<float>((size_t)pl.lists * pl.Np * pl.kc);
-    int32_t* cand_i = wc.take<int32_t>((size_t)pl.lists * pl.Np * pl.kc);
-    int32_t* fb = wc.take<int32_t>(N);
-    float* norms32 = wc.take<float>(pl.Np);
-    float* mu = wc.take<float>(D);
-    int32_t* fb2 = wc.take<int32_t>(N);
-    // two-term stage
-    const bool tt = pl.bf16 && pl.two_term;
-    const size_t nd_s = tt ? (size_t)pl.Np * pl.Dp : 0, np_s = tt ? (size_t)pl.Np : 0;
-    const size_t fd_s = tt ? (size_t)pl.fcap * pl.Dp : 0, f_s = tt ? (size_t)pl.fcap : 0;
-    __nv_bfloat16* xl16 = wc.take<__nv_bfloat16>(nd_s);
-    float* norms_s = wc.take<float>(np_s);
-    float* rho_s = wc.take<float>(np_s);
-    __nv_bfloat16* qh = wc.take<__nv_bfloat16>(fd_s);
-    __nv_bfloat16* ql = wc.take<__nv_bfloat16>(fd_s);
-    float* qnorm = wc.take<float>(f_s);
-    float* scand_d = wc.take<float>(tt ? (size_t)pl.slists * pl.fcap * 32 : 0);
-    int32_t* scand_i = wc.take<int32_t>(tt ? (size_t)pl.slists * pl.fcap * 32 : 0);
-    int32_t* fb3 = wc.take<int32_t>(pl.bf16 ? (size_t)N : 0);
-    __nv_bfloat16* aug = wc.take<__nv_bfloat16>(pl.aug ? 32 * (size_t)pl.Np : 0);
+    const KnnBufs kb = carve_knn(wc, pl, N, D);
+    double* colsum = kb.colsum;
+    void* xt = kb.xt;
+    float *norms = kb.norms, *rho = kb.rho, *cand_d = kb.cand_d, *norms32 = kb.norms32, *mu = kb.mu;
+    int32_t *cand_i = kb.cand_i, *fb = kb.fb, *fb2 = kb.fb2;
+    __nv_bfloat16* aug = kb.aug;
     cudaStream_t s = ctx->stream;
 
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(colsum, 0, sizeof(double) * D, s));
@@ -1721,24 +2004,57 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
         const slk_status r = launch_prep(ctx, X, N, D, pl.Dp, pl.Np, colsum, mu,
                                          pl.bf16 ? nullptr : (float*)xt,
                                          pl.bf16 ? (__nv_bfloat16*)xt : nullptr, norms, rho,
-                                         pl.bf16 ? norms32 : nullptr, pl.aug ? aug : nullptr, st);
+                                         pl.bf16 ? norms32 : nullptr, pl.aug ? aug : nullptr,
+                                         pl.grouped ? &kb.grp : nullptr, st);
         if (r != SLK_OK) return r;
     }
-    float u_acc;   // rounding unit of a tile's dot-product accumulation
+    // rounding unit of a tile's dot-product accumulation: 2^-23 on the tensor
+    // cores (products exact, each accumulator add off by at most one ulp,
+    // truncating; an assumption), 2^-24 for float32
+    const double u_acc = pl.bf16 ? 1.1920928955078125e-07 : 5.9604644775390625e-08;
+    // folded norms: 6 more products a dot, and the aug terms' magnitudes
+    // (about (n_p + n_q) / 2) join the products' sum: 2 |p| |q| + n_p +
+    // n_q = (|p| + |q|)^2, so the bound keeps its form with a 1.01 factor
+    const double g_dot = (double)(pl.Dp + (pl.aug ? 6 : 0)) * u_acc;
+    const double gam = (pl.aug ? 1.01 : 1.0) * g_dot / (1.0 - g_dot);
+    SweepWork work{};
+    work.per = work.n_tiles = pl.n_tiles;
+    work.row_blocks = pl.row_blocks;
+    work.units = pl.units;
+    work.aligned = pl.aligned;
+    const SweepLists lists{reinterpret_cast<uint2*>(cand_d), pl.stride};
     {
-    PhaseScope ps(ctx, SLK_PHASE_KNN_CAND);
-    SLK_COUNT_LAUNCH(ctx, 1);
-    if (pl.bf16) {
-        slk_status r = knn_cand_bf16_launch(ctx, (const __nv_bfloat16*)xt, norms,
-                                            pl.aug ? aug : nullptr, N, pl.Dp, pl.Np, pl.kc, pl.ew,
-                                            pl.splits, cand_d, cand_i, &st->knn_error,
-                                            &st->knn_sweep);
-        if (r != SLK_OK) return r;
-        // 2^-23: products exact, each accumulator add off by at most one ulp
-        // (truncating adds); an assumption about the tensor-core accumulator
-        u_acc = 1.1920928955078125e-07f;
-    } else {
-        u_acc = 5.9604644775390625e-08f;  // 2^-24
+        PhaseScope ps(ctx, SLK_PHASE_KNN_CAND);
+        SLK_COUNT_LAUNCH(ctx, 1);
+        if (pl.bf16) {
+            SweepOperands op{};
+            op.a_hi = op.b_hi = (const __nv_bfloat16*)xt;
+            op.aug = aug;
+            op.row_norms = op.col_norms = norms;
+            op.rho = rho;
+            op.a_rows = op.b_rows = pl.Np;
+            op.N = N;
+            op.D = D;
+            op.Dp = pl.Dp;
+            slk_status r;
+            if (pl.grouped) {
+                // the tiles around each block, then those that can still matter
+                SweepWork first = work;
+                first.per = group_window(pl.n_tiles);
+                first.aligned = 1;
+                r = knn_sweep_launch(ctx, op, first, k, gam, lists, false, kb.grp.thr, kb.grp.kth, st);
+                if (r != SLK_OK) return r;
+                r = group_tiles_launch(ctx, kb.grp, (const __nv_bfloat16*)xt, N, pl.Np, pl.Dp, first);
+                if (r != SLK_OK) return r;
+                SLK_COUNT_LAUNCH(ctx, 1);
+                work.tiles = kb.grp.tiles;
+                work.start = kb.grp.start;
+                work.max_cnt = kb.grp.max_cnt;
+            }
+            r = knn_sweep_launch(ctx, op, work, k, gam, lists, pl.grouped, nullptr,
+                                 pl.grouped ? kb.grp.kth : nullptr, st);
+            if (r != SLK_OK) return r;
+        } else {
 #define SLK_CAND(KC_)                                                                         \
     {                                                                                         \
         auto kern = knn_cand_fp32_kernel<KC_>;                                                \
@@ -1747,44 +2063,54 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
         kern<<<dim3((unsigned)pl.row_blocks, (unsigned)pl.splits), KT, smem, s>>>(            \
             (const float*)xt, norms, N, pl.Dp, pl.n_tiles, pl.Np, cand_d, cand_i);            \
     }
-        if (pl.kc == 16) SLK_CAND(16) else SLK_CAND(32)
+            if (pl.kc == 16) SLK_CAND(16) else SLK_CAND(32)
 #undef SLK_CAND
-        SLK_LAUNCH_CHECK(ctx, "knn_cand_fp32_kernel");
+            SLK_LAUNCH_CHECK(ctx, "knn_cand_fp32_kernel");
+        }
     }
-    }
+    SelectArgs sel{};
+    sel.X = X;
+    sel.N = N;
+    sel.D = D;
+    sel.Dp = pl.Dp;
+    sel.k = k;
+    sel.row_ptr = row_ptr;
+    sel.col_idx = col_idx;
+    sel.dist2 = dist2;
+    sel.st = st;
     {
         PhaseScope ps(ctx, SLK_PHASE_KNN_RERANK);
         SLK_COUNT_LAUNCH(ctx, 1);
         int64_t grid = (N + 7) / 8;
         if (grid > (int64_t)ctx->num_sms * 16) grid = (int64_t)ctx->num_sms * 16;
+        if (pl.bf16) {
+            sel.w = work;
+            sel.lists = lists;
+            sel.perm = pl.grouped ? kb.grp.perm : nullptr;
+            sel.norms = norms;
+            sel.rho = rho;
+            sel.gam = gam;
+            sel.fb_list = fb;
+            sel.fb_count = (unsigned long long*)&st->fallback_count;
+            knn_select_kernel<false><<<(unsigned)grid, 256, 0, s>>>(sel);
+            SLK_LAUNCH_CHECK(ctx, "knn_select_kernel");
+        } else {
         // entries per lane: the splits' lists, KC each, over 32 lanes
-        const int per_lane = (pl.lists * pl.kc + 31) / 32;
-        // folded norms: 6 more products a dot, and the aug terms' magnitudes
-        // (about (n_p + n_q) / 2) join the products' sum: 2 |p| |q| + n_p +
-        // n_q = (|p| + |q|)^2, so the bound keeps its form with a 1.01 factor
-        const double g = (double)(pl.Dp + (pl.aug ? 6 : 0)) * (double)u_acc;
-        const double gam = (pl.aug ? 1.01 : 1.0) * g / (1.0 - g);
+        const int per_lane = (pl.splits * pl.kc + 31) / 32;
 #define SLK_RERANK(KC_, E_)                                                                   \
-    do {                                                                                      \
-        if (pl.kc == 32 && pl.ew == 8)                                                        \
-            knn_rerank_kernel<32, 0, E_, 64><<<(unsigned)grid, 256, 0, s>>>(                  \
-                X, N, D, pl.Dp, k, pl.lists, pl.Np, cand_d, cand_i, norms, rho, gam, row_ptr,   \
-                col_idx, dist2, fb, st);                                                      \
-        else                                                                                  \
-            knn_rerank_kernel<KC_, 0, E_><<<(unsigned)grid, 256, 0, s>>>(                     \
-                X, N, D, pl.Dp, k, pl.lists, pl.Np, cand_d, cand_i, norms, rho, gam, row_ptr,   \
-                col_idx, dist2, fb, st);                                                      \
-    } while (0)
+    knn_rerank_kernel<KC_, 0, E_><<<(unsigned)grid, 256, 0, s>>>(                             \
+        X, N, D, pl.Dp, k, pl.splits, pl.Np, cand_d, cand_i, norms, rho, gam, row_ptr, col_idx, \
+        dist2, fb, st)
 #define SLK_RERANK_E(KC_)                                                                     \
     if (per_lane <= 4) SLK_RERANK(KC_, 4);                                                    \
     else if (per_lane <= 8) SLK_RERANK(KC_, 8);                                               \
     else SLK_RERANK(KC_, 16);
         if (pl.kc == 16) { SLK_RERANK_E(16) }
-        else if (pl.kc == 32) { SLK_RERANK_E(32) }
-        else { SLK_RERANK_E(64) }
+        else { SLK_RERANK_E(32) }
 #undef SLK_RERANK_E
 #undef SLK_RERANK
         SLK_LAUNCH_CHECK(ctx, "knn_rerank_kernel");
+        }
     }
     {
         PhaseScope ps(ctx, SLK_PHASE_KNN_FALLBACK);
@@ -1795,6 +2121,7 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
         if (pl.bf16) {
             // the float32 stage's input and its failures (for the exact scan)
             const int32_t* f32_in = fb;
+            int32_t* fb3 = pl.two_term ? fb : fb2;   // the list that is not its input
             const long long* f32_cnt = &st->fallback_count;
             if (pl.two_term) {
             f32_in = fb2;
@@ -1808,48 +2135,64 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
             int64_t pg = (pl.Np + 7) / 8;
             if (pg > (int64_t)ctx->num_sms * 64) pg = (int64_t)ctx->num_sms * 64;
             SLK_COUNT_LAUNCH(ctx, 4);
+            // the operand back in the points' order where the sweep had sorted it
+            __nv_bfloat16* xh = pl.grouped ? (__nv_bfloat16*)xt : nullptr;
             if (v4)
                 prep_split_kernel<4><<<(unsigned)pg, 256, 0, s>>>(X, N, D, pl.Dp, pl.Np, mu,
-                                                                  &st->fallback_count, xl16, norms_s,
-                                                                  rho_s, st);
+                                                                  &st->fallback_count, xh, kb.xl16,
+                                                                  kb.norms_s, kb.rho_s, st);
             else
                 prep_split_kernel<1><<<(unsigned)pg, 256, 0, s>>>(X, N, D, pl.Dp, pl.Np, mu,
-                                                                  &st->fallback_count, xl16, norms_s,
-                                                                  rho_s, st);
+                                                                  &st->fallback_count, xh, kb.xl16,
+                                                                  kb.norms_s, kb.rho_s, st);
             SLK_LAUNCH_CHECK(ctx, "prep_split_kernel");
             int64_t gg = (pl.fcap + 7) / 8;
             if (gg > (int64_t)ctx->num_sms * 16) gg = (int64_t)ctx->num_sms * 16;
-            gather_split_kernel<<<(unsigned)gg, 256, 0, s>>>((const __nv_bfloat16*)xt, xl16, norms_s,
+            gather_split_kernel<<<(unsigned)gg, 256, 0, s>>>((const __nv_bfloat16*)xt, kb.xl16, kb.norms_s,
                                                             pl.Dp, fb, &st->fallback_count, pl.fcap,
-                                                            qh, ql, qnorm);
+                                                            kb.qh, kb.ql, kb.qnorm);
             SLK_LAUNCH_CHECK(ctx, "gather_split_kernel");
-            slk_status r = knn_cand_split_launch(ctx, qh, ql, qnorm, pl.fcap, &st->fallback_count,
-                                                 (const __nv_bfloat16*)xt, xl16, norms_s, N, pl.Dp,
-                                                 pl.Np, pl.ew, pl.ssplits, scand_d, scand_i,
-                                                 &st->knn_error);
+            // dot products of 3 Dp bfloat16 products (2^-23 accumulator
+            // unit, as above), |h|, |l| within 1.004 |s| and 0.0040 |s|,
+            // plus the dropped l . l term (at most 1.016 2^-16 |s_p| |s_q|)
+            const double g3 = 3.0 * (double)pl.Dp * 1.1920928955078125e-07;
+            const double gam_s = 1.02 * g3 / (1.0 - g3) + 1.02 * 1.52587890625e-05;
+            SweepOperands op{};
+            op.a_hi = kb.qh;
+            op.a_lo = kb.ql;
+            op.b_hi = (const __nv_bfloat16*)xt;
+            op.b_lo = kb.xl16;
+            op.row_norms = kb.qnorm;
+            op.col_norms = kb.norms_s;
+            op.rho = kb.rho_s;
+            op.ids = fb;
+            op.rows_dev = &st->fallback_count;
+            op.a_rows = pl.fcap;
+            op.b_rows = pl.Np;
+            op.N = N;
+            op.D = D;
+            op.Dp = pl.Dp;
+            SweepWork swork{};
+            swork.per = swork.n_tiles = pl.n_tiles;
+            swork.row_blocks = (int)(pl.fcap / 128);
+            swork.units = pl.sunits;
+            swork.aligned = 0;
+            const SweepLists slists{kb.scand, kSweepStride};
+            slk_status r = knn_sweep_launch(ctx, op, swork, k, gam_s, slists, false, nullptr, nullptr, st);
             if (r != SLK_OK) return r;
-            {
-                // dot products of 3 Dp bfloat16 products (2^-23 accumulator
-                // unit, as above), |h|, |l| within 1.004 |s| and 0.0040 |s|,
-                // plus the dropped l . l term (at most 1.016 2^-16 |s_p| |s_q|)
-                const double g3 = 3.0 * (double)pl.Dp * 1.1920928955078125e-07;
-                const double gam_s = 1.02 * g3 / (1.0 - g3) + 1.02 * 1.52587890625e-05;
-                const unsigned rgrid = (unsigned)(ctx->num_sms * 4);
-                const int per_lane = (pl.slists * 32 + 31) / 32;
-#define SLK_RERANK_S(E_, SEL_)                                                                \
-    knn_rerank_kernel<32, 2, E_, SEL_><<<rgrid, 256, 0, s>>>(                                 \
-        X, N, D, pl.Dp, k, pl.slists, pl.fcap, scand_d, scand_i, norms_s, rho_s, gam_s, row_ptr, \
-        col_idx, dist2, fb2, st, fb, &st->fallback_count, &st->fallback2_count)
-                if (pl.ew == 8) {
-                    if (per_lane <= 8) SLK_RERANK_S(8, 64);
-                    else SLK_RERANK_S(16, 64);
-                } else {
-                    if (per_lane <= 8) SLK_RERANK_S(8, 32);
-                    else SLK_RERANK_S(16, 32);
-                }
-#undef SLK_RERANK_S
-                SLK_LAUNCH_CHECK(ctx, "knn_rerank_kernel (two-term stage)");
-            }
+            sel.w = swork;
+            sel.lists = slists;
+            sel.perm = nullptr;
+            sel.norms = kb.norms_s;
+            sel.rho = kb.rho_s;
+            sel.gam = gam_s;
+            sel.fb_list = fb2;
+            sel.fb_count = (unsigned long long*)&st->fallback2_count;
+            sel.fb_in = fb;
+            sel.count_in = &st->fallback_count;
+            sel.cap = pl.fcap;
+            knn_select_kernel<true><<<(unsigned)(ctx->num_sms * 4), 256, 0, s>>>(sel);
+            SLK_LAUNCH_CHECK(ctx, "knn_select_kernel (two-term stage)");
             }
             // (b) float32 distance tiles of the rows still open against every
             // point, then the rerank under the float32 certificate; its
@@ -1857,7 +2200,7 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
             // between the k-th and the last decides the certificate)
             const int kcq = (2 * k <= 16) ? 16 : 32;
             // column splits chosen on the device from the count (query_splits)
-            const long long qcap = (long long)pl.lists * pl.Np * pl.kc;
+            const long long qcap = (long long)cand_floats(pl);
             const int n_tiles = (int)((N + BN - 1) / BN);
             SLK_COUNT_LAUNCH(ctx, 2);
             const unsigned qgrid = (unsigned)(ctx->num_sms * 2);
@@ -1890,7 +2233,7 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
         // the batched rescan's partial lists reuse the candidate buffer
         // (its lists are read by now): cs column ranges of k entries for each
         // of the F open rows, cs chosen on the device from F
-        const long long cap = (long long)pl.lists * pl.Np * pl.kc;
+        const long long cap = (long long)cand_floats(pl);
         const int dpl = (D + 31) / 32;
         if (dpl <= 32) {
             SLK_COUNT_LAUNCH(ctx, 2);

@@ -731,7 +731,7 @@ extern "C" slk_status slk_server_submit(slk_server* sv, const slk_instance* q, i
     if (q->N < 2 || q->N >= (int64_t)0x7fffffff || q->D < 1 || q->L < 1 || q->L > SLK_BATCH_MAX_L ||
         q->L > q->N || q->k < 1 || q->k > SLK_MAX_K || q->k > q->N - 1)
         return set_err(ctx, SLK_ERR_INVALID_ARG, "request: bad sizes");
-    const size_t need = request_bytes(sv, *q) + knn_ws_bytes(ctx, q->N, q->D, q->k, sv->p.knn_precision);
+    const size_t need = request_bytes(sv, *q) + knn_ws_min_bytes(ctx, q->N, q->D, q->k, sv->p.knn_precision);
     if (need > sv->arena_bytes)
         return set_err(ctx, SLK_ERR_OOM, "request needs %zu bytes, the server arena has %zu", need,
                        sv->arena_bytes);
@@ -747,7 +747,7 @@ extern "C" slk_status slk_server_submit(slk_server* sv, const slk_instance* q, i
 extern "C" slk_status slk_server_request_bytes(slk_server* sv, const slk_instance* q, int64_t* bytes) {
     if (!sv || !q || !bytes) return SLK_ERR_INVALID_ARG;
     *bytes = (int64_t)(align_up(request_bytes(sv, *q), 256) +
-                       align_up(knn_ws_bytes(sv->ctx, q->N, q->D, q->k, sv->p.knn_precision), 256));
+                       align_up(knn_ws_min_bytes(sv->ctx, q->N, q->D, q->k, sv->p.knn_precision), 256));
     return SLK_OK;
 }
 
@@ -773,9 +773,14 @@ slk_status admit(slk_server* sv, int64_t id) {
     if (slot < 0) return SLK_ERR_OOM;
     Block mem, scr;
     if (!arena_alloc(sv, request_bytes(sv, q), mem)) return SLK_ERR_OOM;
-    if (!arena_alloc(sv, knn_ws_bytes(ctx, q.N, q.D, q.k, sv->p.knn_precision), scr)) {
-        arena_free(sv, mem);
-        return SLK_ERR_OOM;
+    // the graph's scratch: as much as it works best with, or the least it needs
+    size_t knn_bytes = knn_ws_bytes(ctx, q.N, q.D, q.k, sv->p.knn_precision);
+    if (!arena_alloc(sv, knn_bytes, scr)) {
+        knn_bytes = knn_ws_min_bytes(ctx, q.N, q.D, q.k, sv->p.knn_precision);
+        if (!arena_alloc(sv, knn_bytes, scr)) {
+            arena_free(sv, mem);
+            return SLK_ERR_OOM;
+        }
     }
     r.slot = slot;
     r.mem = mem;
@@ -827,7 +832,7 @@ slk_status admit(slk_server* sv, int64_t id) {
     ctx->stream = sv->aux[r.aux];
     DevState* st = sv->aux_st + r.aux;
     slk_status rs = knn_graph_launch(ctx, q.X, q.N, q.D, q.k, sv->p.knn_precision, row_ptr, col, dist2,
-                                     sv->arena + scr.off, st);
+                                     sv->arena + scr.off, knn_bytes, st);
     if (rs == SLK_OK)
         rs = (q.sigma > 0.f) ? set_sigma_launch(ctx, q.sigma, st)
                              : sigma_launch(ctx, dist2, q.N * (int64_t)q.k, sv->p.sigma_rule, st);

@@ -21,6 +21,7 @@ struct slk_ctx {
     // scratch workspace, grown on demand (cudaMalloc), freed by slk_destroy
     void* ws = nullptr;
     size_t ws_bytes = 0;
+    size_t ws_refused = SIZE_MAX;   // smallest size that could not be allocated
     // small pinned host block for scalar results
     void* host_pin = nullptr;
     // small device block for scalar state (status words, sigma, energy)
@@ -103,6 +104,9 @@ slk_status set_err(slk_ctx* ctx, slk_status st, const char* fmt, ...);
 slk_status cuda_err(slk_ctx* ctx, cudaError_t e, const char* where);
 // Make sure ctx->ws holds at least `bytes`; returns SLK_OK or SLK_ERR_OOM.
 slk_status ensure_ws(slk_ctx* ctx, size_t bytes);
+// The same for `want` bytes, or for `least` where so much cannot be had (asked
+// for only once per size); *full: whether there are `want`.
+slk_status ensure_ws_of(slk_ctx* ctx, size_t want, size_t least, bool* full);
 
 #define SLK_CUDA_TRY(ctx, expr)                                                  \
     do {                                                                         \
@@ -132,12 +136,14 @@ struct WsCarver {
     }
 };
 
-// Workspace needed by knn_graph_launch (bytes), and the launcher itself
-// (device outputs only; no synchronisation).
+// Workspace knn_graph_launch works best with (bytes) and the least it needs,
+// and the launcher itself (device outputs only; no synchronisation), which
+// makes its plan from the bytes it is given.
 size_t knn_ws_bytes(const slk_ctx* ctx, int64_t N, int D, int k, int precision);
+size_t knn_ws_min_bytes(const slk_ctx* ctx, int64_t N, int D, int k, int precision);
 slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int k,
                             int precision, int64_t* row_ptr, int32_t* col_idx, float* dist2,
-                            void* ws, DevState* st);
+                            void* ws, size_t ws_bytes, DevState* st);
 
 // Centred float32 operand of the distance tiles: xt[p][j] = x_pj - mean_j
 // (Np x Dp, zero padding), norms[p] = ||xt_p||^2, rho[p] = rounding norm.
