@@ -9,9 +9,20 @@
 //                        stable counting sort of the points by cluster
 //                        (perm, offsets), deterministic
 //   density_tile_kernel  128 x 128 float32 distance tiles of the centred
-//                        data by the norm expansion, one cluster's columns
-//                        per work item, exp in the epilogue, per-row sums of
-//                        8 kernel values in float32 added in float64
+//                        data by the norm expansion, rows and columns in the
+//                        sorted order, one cluster's columns per work item, exp
+//                        in the epilogue, per-row sums of 8 kernel values in
+//                        float32 added in float64; first every cluster against
+//                        itself, which gives a lower bound T_l of max f_l, then
+//                        the row blocks of other clusters that may still reach
+//                        T_l (density_reach_kernel).  For a row y of cluster j
+//                        and a point p of cluster l, the signed distances
+//                          h_jl(x) = (||x - s_l||^2 - ||x - s_j||^2) / (2 ||s_j - s_l||)
+//                        from the border between the two seeds give ||y - p|| >=
+//                        h_jl(y) + h_lj(p), so a histogram of cluster l's h_lj
+//                        bounds f_l(y) from h_jl(y) alone.  70000 x 784, 10 clusters:
+//                        29.5 ms of tiles (47 TFLOP/s on the float32 units),
+//                        against 154 over all pairs of points
 //   density_bound_kernel / density_cand_kernel
 //                        f^_l(y) = the float64 sum of the items of cluster l;
 //                        the tiles' rounding bounds give |d^2 - d2| <= delta_y,
@@ -42,7 +53,7 @@ constexpr int kSortChunk = 1024;  // points per block of the counting sort
 template <int LPT>
 __global__ void __launch_bounds__(256)
 seed_assign_kernel(const float* __restrict__ X, int64_t N, int D, const int32_t* __restrict__ seeds,
-                   int L, int32_t* __restrict__ assign) {
+                   int L, int32_t* __restrict__ assign, float* __restrict__ d2out) {
     extern __shared__ float sm[];
     float* xs = sm;                   // [32][33]
     float* ss = xs + 32 * 33;         // [L][33]
@@ -86,6 +97,8 @@ seed_assign_kernel(const float* __restrict__ X, int64_t N, int D, const int32_t*
         if (l < L) dd[pl * L + l] = acc[j];
     }
     __syncthreads();
+    for (int i = t; i < 32 * L; i += 256)   // [N][L] distances for the reach bounds
+        if (p0 + i / L < N) d2out[p0 * L + i] = (float)dd[i];
     if (t < 32 && p0 + t < N) {
         int best = 0;
         double bd = dd[t * L];
@@ -199,6 +212,11 @@ struct DensItem {
     int32_t slot;         // row of the partial-sum matrix
 };
 
+// 128 (or fewer) consecutive places of one cluster.
+struct DensRows {
+    int32_t label, row0, row1;
+};
+
 struct DensSmem {
     float As[2][DBK][DBM];
     float Bs[2][DBK][DBN];
@@ -206,25 +224,33 @@ struct DensSmem {
     float nrow[DBM];
     float ncol[DBN];
     int cidx[DBN];
+    int ridx[DBM];
 };
 
-// Grid: (row blocks of 128, items).  Thread (ty, tx) = (t / 16, t % 16) owns
-// rows {4ty..4ty+3, 64+4ty..+3} and the same pattern of columns.
+// Grid: (row blocks, items).  Thread (ty, tx) = (t / 16, t % 16) owns rows
+// {4ty..4ty+3, 64+4ty..+3} and the same pattern of columns.  other: 0 the
+// row blocks of the item's own cluster, 1 those of the others that need it.
 __global__ void __launch_bounds__(DT, 2)
 density_tile_kernel(const float* __restrict__ xt, const float* __restrict__ norms, int64_t N,
-                    int Dp, const int32_t* __restrict__ perm, const DensItem* __restrict__ items,
+                    int Dp, const int32_t* __restrict__ perm, const DensRows* __restrict__ rows,
+                    const DensItem* __restrict__ items, int other, const uint8_t* __restrict__ need, int L,
                     const float* __restrict__ sigma_dev, double* __restrict__ part) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     DensSmem& s = *reinterpret_cast<DensSmem*>(smem_raw);
     const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
-    const int64_t row0 = (int64_t)blockIdx.x * DBM;
+    const DensRows rw = rows[blockIdx.x];
     const DensItem it = items[blockIdx.y];
+    if ((rw.label == it.label) == (other != 0)) return;
+    if (other && !need[(int64_t)blockIdx.x * L + it.label]) return;
     const float sg = *sigma_dev;
     const float inv2s2 = 1.0f / (2.0f * sg * sg);
     if (t < DBM) {
-        s.nrow[t] = norms[row0 + t];
+        const int y = perm[rw.row0 + t < rw.row1 ? rw.row0 + t : rw.row0];
+        s.ridx[t] = y;
+        s.nrow[t] = norms[y];
         s.rowsum[t] = 0.0;
     }
+    __syncthreads();
     const int nk = Dp / DBK;
     const int lr0 = t & 127, lq0 = t >> 7, lq1 = lq0 + 2;
     for (int c0 = it.col0; c0 < it.col1; c0 += DBN) {
@@ -242,7 +268,7 @@ density_tile_kernel(const float* __restrict__ xt, const float* __restrict__ norm
 #pragma unroll
             for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
         const int qb = s.cidx[lr0] >= 0 ? s.cidx[lr0] : s.cidx[0];
-        const float* pa = xt + (row0 + lr0) * Dp;
+        const float* pa = xt + (int64_t)s.ridx[lr0] * Dp;
         const float* pb = xt + (int64_t)qb * Dp;
         float4 ra0 = __ldg(reinterpret_cast<const float4*>(pa + 4 * lq0));
         float4 ra1 = __ldg(reinterpret_cast<const float4*>(pa + 4 * lq1));
@@ -310,7 +336,74 @@ density_tile_kernel(const float* __restrict__ xt, const float* __restrict__ norm
         }
     }
     __syncthreads();
-    if (t < DBM && row0 + t < N) part[(int64_t)it.slot * N + row0 + t] = s.rowsum[t];
+    if (t < DBM && rw.row0 + t < rw.row1) part[(int64_t)it.slot * N + s.ridx[t]] = s.rowsum[t];
+}
+
+// Depth of the points of each row block (cluster j) behind the border toward
+// every seed l: lo[b][l] = min_y h_jl(y), and hist[j][l], the cluster's points
+// by their depth in quarters of sigma (place k: at least (k - 32) / 4 sigma,
+// place 0: nothing is known).  d2 [N][L]: squared distances to the seeds
+// (within 4e-6).
+constexpr int kDepthBins = 64;
+__global__ void __launch_bounds__(DBM)
+density_depth_kernel(const float* __restrict__ d2, const int32_t* __restrict__ perm,
+                     const DensRows* __restrict__ rows, const int32_t* __restrict__ seeds, int L,
+                     const float* __restrict__ sigma_dev, float* __restrict__ lo, int* __restrict__ hist) {
+    __shared__ float wm[DBM / 32];
+    __shared__ int bins[kDepthBins];
+    const DensRows rw = rows[blockIdx.x];
+    const int t = threadIdx.x, j = rw.label;
+    const bool in = rw.row0 + t < rw.row1;
+    const int64_t y = perm[in ? rw.row0 + t : rw.row0];
+    const float dj = d2[y * L + j], inv = 4.f / *sigma_dev;
+    if (t < kDepthBins) bins[t] = 0;
+    __syncthreads();
+    for (int l = 0; l < L; ++l) {
+        const float dl = d2[y * L + l], ds = d2[(int64_t)seeds[l] * L + j];
+        float h = -__int_as_float(0x7f800000);   // no border: nothing is known
+        if (l != j && ds > 1e-20f) h = (dl - dj - 4e-6f * (dl + dj)) / (2.00001f * sqrtf(ds));
+        if (h < 0.f) h *= 1.0001f;
+        if (in) {
+            const float k = fminf(floorf(h * inv), (float)(kDepthBins - 33));   // at most the last place
+            atomicAdd(&bins[k > -32.f ? (int)k + 32 : 0], 1);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) h = fminf(h, __shfl_xor_sync(0xffffffffu, h, o));
+        if ((t & 31) == 0) wm[t >> 5] = h;
+        __syncthreads();
+        if (t == 0) {
+            for (int w = 1; w < DBM / 32; ++w) h = fminf(h, wm[w]);
+            lo[(int64_t)blockIdx.x * L + l] = h;
+        }
+        if (t < kDepthBins) {
+            if (bins[t]) atomicAdd(&hist[((int64_t)j * L + l) * kDepthBins + t], bins[t]);
+            bins[t] = 0;
+        }
+        __syncthreads();
+    }
+}
+
+// need[b][l]: a row of block b (another cluster's) may reach T_l:
+// f_l(y) <= sum over cluster l's depths of exp(-(h_jl(y) + h_lj(p))^2 / 2 sigma^2).
+__global__ void __launch_bounds__(256)
+density_reach_kernel(const float* __restrict__ lo, const int* __restrict__ hist,
+                     const DensRows* __restrict__ rows, int n_rows, int L,
+                     const unsigned long long* __restrict__ tbits, const float* __restrict__ sigma_dev,
+                     uint8_t* __restrict__ need) {
+    const float inv = 1.f / *sigma_dev;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < (int64_t)n_rows * L;
+         i += (int64_t)gridDim.x * 256) {
+        const int b = (int)(i / L), l = (int)(i % L), j = rows[b].label;
+        const double T = __longlong_as_double((long long)tbits[l]);
+        const int* h = hist + ((int64_t)l * L + j) * kDepthBins;
+        const float y = lo[i] * inv;
+        float f = (float)h[0];
+        for (int k = 1; k < kDepthBins; ++k) {
+            const float r = fmaxf(y + 0.25f * (float)(k - 32) - 1e-4f, 0.f) * 0.9999f;
+            f += (float)h[k] * expf(-0.5f * r * r);
+        }
+        need[i] = !((double)f * 1.0001 < T);   // NaN (no border) needs it
+    }
 }
 
 // f^_l(y): the item rows of label l summed in slot order.
@@ -371,14 +464,16 @@ density_bound_kernel(const double* __restrict__ part, int64_t N, int Dp,
     }
 }
 
-// f_l(y) of candidate c (or, with all_pairs, of pair c = y L + l) from the
-// features: 8 warps over the points of cluster l, warp_sq_dist distances,
-// float64 kernel sums in a fixed order.
+// Part blockIdx.y of f_l(y) of candidate c (or, with all_pairs, of pair c = y L +
+// l) from the features: its share of the points of cluster l, 8 warps,
+// warp_sq_dist distances, float64 kernel sums in a fixed order.  A handful of
+// candidates is the usual case (11 at 70000 x 784): one block each took 2.6 ms,
+// split over the GPU 0.13 ms.
 __global__ void __launch_bounds__(256)
 density_exact_kernel(const float* __restrict__ X, int64_t N, int D, int L,
                      const int32_t* __restrict__ perm, const int64_t* __restrict__ off,
                      const int2* __restrict__ cand, int all_pairs, int64_t c0,
-                     const float* __restrict__ sigma_dev, double* __restrict__ fexact) {
+                     const float* __restrict__ sigma_dev, double* __restrict__ fpart) {
     __shared__ double red[8];
     const int64_t c = c0 + blockIdx.x;
     int64_t y;
@@ -394,8 +489,10 @@ density_exact_kernel(const float* __restrict__ X, int64_t N, int D, int L,
     const double sg = (double)*sigma_dev;
     const double inv2s2 = 1.0 / (2.0 * sg * sg);
     const float* xy = X + y * D;
+    const int64_t n = off[l + 1] - off[l];
+    const int64_t i0 = off[l] + n * blockIdx.y / gridDim.y, i1 = off[l] + n * (blockIdx.y + 1) / gridDim.y;
     double f = 0.0;
-    for (int64_t i = off[l] + warp; i < off[l + 1]; i += 8) {
+    for (int64_t i = i0 + warp; i < i1; i += 8) {
         const int64_t p = perm[i];
         const double d2 = warp_sq_dist(X + p * D, xy, nullptr, D, lane);
         f += exp(-d2 * inv2s2);
@@ -405,14 +502,14 @@ density_exact_kernel(const float* __restrict__ X, int64_t N, int D, int L,
     if (threadIdx.x == 0) {
         double s = 0.0;
         for (int w = 0; w < 8; ++w) s += red[w];
-        fexact[blockIdx.x] = s;
+        fpart[(int64_t)blockIdx.x * gridDim.y + blockIdx.y] = s;
     }
 }
 
 // Pass 0: the largest exact density per label (non-negative doubles order as
 // their bit patterns); pass 1: the smallest y attaining it.
 __global__ void __launch_bounds__(256)
-density_pick_kernel(const double* __restrict__ fexact, const int2* __restrict__ cand, int64_t c0,
+density_pick_kernel(const double* __restrict__ fpart, int parts, const int2* __restrict__ cand, int64_t c0,
                     int64_t count, int all_pairs, int L, int pass,
                     unsigned long long* __restrict__ fmax_bits, int32_t* __restrict__ arg) {
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < count;
@@ -420,7 +517,9 @@ density_pick_kernel(const double* __restrict__ fexact, const int2* __restrict__ 
         const int64_t c = c0 + i;
         const int64_t y = all_pairs ? c / L : cand[c].x;
         const int l = all_pairs ? (int)(c % L) : cand[c].y;
-        const unsigned long long fb = (unsigned long long)__double_as_longlong(fexact[i]);
+        double f = 0.0;
+        for (int q = 0; q < parts; ++q) f += fpart[i * parts + q];
+        const unsigned long long fb = (unsigned long long)__double_as_longlong(f);
         if (pass == 0) atomicMax(&fmax_bits[l], fb);
         else if (fb == fmax_bits[l]) atomicMin(&arg[l], (int)y);
     }
@@ -444,6 +543,7 @@ struct InitPlan {
     int Dp, nb;       // padded sizes, sort blocks
     int chunk;        // columns per density item (multiple of 128)
     int max_items;
+    int max_rows;     // row blocks of 128 places, cut at the clusters
     int64_t cand_cap; // candidates kept in a list; more means every (y, l) is recomputed
 };
 
@@ -457,6 +557,7 @@ InitPlan init_plan(int64_t N, int D, int L) {
     if (per < 16) per = 16;
     p.chunk = (int)(per * DBN);
     p.max_items = (int)((N + p.chunk - 1) / p.chunk) + L;
+    p.max_rows = (int)(tiles + L);
     p.cand_cap = std::min<int64_t>((int64_t)N * L, (int64_t)1 << 22);
     return p;
 }
@@ -480,6 +581,9 @@ size_t init_modes_ws_bytes(const slk_ctx* ctx, int64_t N, int D, int L) {
     b += align_up(sizeof(int2) * (size_t)p.cand_cap, 256);                 // candidates
     b += align_up(sizeof(double) * (size_t)p.cand_cap, 256);               // exact densities
     b += align_up(sizeof(unsigned long long) * (L + 2), 256);             // T_l, count
+    b += align_up(sizeof(DensRows) * p.max_rows, 256) + align_up((size_t)p.max_rows * L, 256);
+    b += align_up(sizeof(float) * (size_t)p.max_rows * L, 256) +
+         align_up(sizeof(int) * kDepthBins * (size_t)L * L, 256);
     return b + 4096;
 }
 
@@ -507,6 +611,13 @@ slk_status init_modes_launch(slk_ctx* ctx, const float* X, int64_t N, int D, con
     double* fexact = wc.take<double>((size_t)pl.cand_cap);
     unsigned long long* tbits = wc.take<unsigned long long>(L + 2);
     unsigned long long* ncand = tbits + L;
+    DensRows* rows = wc.take<DensRows>(pl.max_rows);
+    uint8_t* need = wc.take<uint8_t>((size_t)pl.max_rows * L);
+    float* lo = wc.take<float>((size_t)pl.max_rows * L);
+    int* hist = wc.take<int>((size_t)L * L * kDepthBins);
+    // the distances to the seeds live in the partial sums' place until those
+    // are cleared (max_items >= L doubles a point)
+    float* d2 = reinterpret_cast<float*>(part);
 
     // 1. nearest seed
     {
@@ -519,7 +630,7 @@ slk_status init_modes_launch(slk_ctx* ctx, const float* X, int64_t N, int D, con
         auto kern = seed_assign_kernel<LPT_>;                                                   \
         SLK_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                                (int)smem));                                     \
-        kern<<<grid, 256, smem, s>>>(X, N, D, seeds, L, assign);                                \
+        kern<<<grid, 256, smem, s>>>(X, N, D, seeds, L, assign, d2);                                \
     }
         if (lpt <= 1) { SLK_ASSIGN(1) }
         else if (lpt <= 2) { SLK_ASSIGN(2) }
@@ -560,24 +671,39 @@ slk_status init_modes_launch(slk_ctx* ctx, const float* X, int64_t N, int D, con
                                       cudaMemcpyHostToDevice, s));
     SLK_CUDA_TRY(ctx, cudaMemcpyAsync(slot0, hslot.data(), sizeof(int32_t) * (L + 1),
                                       cudaMemcpyHostToDevice, s));
-    // 5. density tiles
-    if (!hit.empty()) {
-        SLK_COUNT_LAUNCH(ctx, 1);
-        const int smem = (int)sizeof(DensSmem);
-        SLK_CUDA_TRY(ctx, cudaFuncSetAttribute(density_tile_kernel,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        density_tile_kernel<<<dim3((unsigned)(pl.Np / DBM), (unsigned)hit.size()), DT, smem, s>>>(
-            xt, norms, N, pl.Dp, perm, items, sigma_dev, part);
-        SLK_LAUNCH_CHECK(ctx, "density_tile_kernel");
-    }
-    // 6. candidates: upper bound of f_l(y) reaches the largest lower bound
-    SLK_COUNT_LAUNCH(ctx, 2);
+    std::vector<DensRows> hrow;
+    for (int l = 0; l < L; ++l)
+        for (int64_t c = hoff[l]; c < hoff[l + 1]; c += DBM)
+            hrow.push_back({l, (int32_t)c, (int32_t)std::min<int64_t>(c + DBM, hoff[l + 1])});
+    const int n_rows = (int)hrow.size();
+    if (n_rows > pl.max_rows) return set_err(ctx, SLK_ERR_CUDA, "density rows overflow");
+    SLK_CUDA_TRY(ctx, cudaMemcpyAsync(rows, hrow.data(), sizeof(DensRows) * hrow.size(),
+                                      cudaMemcpyHostToDevice, s));
+    // 5. density tiles: own clusters, T_l, then the row blocks that may reach it
+    SLK_CUDA_TRY(ctx, cudaMemsetAsync(hist, 0, sizeof(int) * (size_t)L * L * kDepthBins, s));
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(tbits, 0, sizeof(unsigned long long) * (L + 1), s));
     int gx = (int)((N + 255) / 256);
     if (gx > 4 * ctx->num_sms) gx = 4 * ctx->num_sms;
+    const int smem = (int)sizeof(DensSmem);
+    SLK_CUDA_TRY(ctx, cudaFuncSetAttribute(density_tile_kernel,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const dim3 tgrid((unsigned)n_rows, (unsigned)hit.size()), bgrid((unsigned)gx, (unsigned)L);
+    SLK_COUNT_LAUNCH(ctx, 7);
+    density_depth_kernel<<<(unsigned)n_rows, DBM, 0, s>>>(d2, perm, rows, seeds, L, sigma_dev, lo, hist);
+    SLK_CUDA_TRY(ctx, cudaMemsetAsync(part, 0, sizeof(double) * hit.size() * (size_t)N, s));
+    density_tile_kernel<<<tgrid, DT, smem, s>>>(xt, norms, N, pl.Dp, perm, rows, items, 0, need, L,
+                                                sigma_dev, part);
+    density_bound_kernel<<<bgrid, 256, 0, s>>>(part, N, pl.Dp, norms, st, sigma_dev, slot0, 0, tbits, cand,
+                                               ncand, pl.cand_cap);
+    density_reach_kernel<<<(unsigned)gx, 256, 0, s>>>(lo, hist, rows, n_rows, L, tbits, sigma_dev, need);
+    density_tile_kernel<<<tgrid, DT, smem, s>>>(xt, norms, N, pl.Dp, perm, rows, items, 1, need, L,
+                                                sigma_dev, part);
+    SLK_LAUNCH_CHECK(ctx, "density_tile_kernel");
+    // 6. candidates: upper bound of f_l(y) reaches the largest lower bound (a
+    // sum that was left out is 0 and cannot)
     for (int pass = 0; pass < 2; ++pass)
-        density_bound_kernel<<<dim3((unsigned)gx, (unsigned)L), 256, 0, s>>>(
-            part, N, pl.Dp, norms, st, sigma_dev, slot0, pass, tbits, cand, ncand, pl.cand_cap);
+        density_bound_kernel<<<bgrid, 256, 0, s>>>(part, N, pl.Dp, norms, st, sigma_dev, slot0, pass, tbits,
+                                                   cand, ncand, pl.cand_cap);
     SLK_LAUNCH_CHECK(ctx, "density_bound_kernel");
     unsigned long long hcount = 0;
     SLK_CUDA_TRY(ctx, cudaMemcpyAsync(&hcount, ncand, sizeof(hcount), cudaMemcpyDeviceToHost, s));
@@ -588,18 +714,22 @@ slk_status init_modes_launch(slk_ctx* ctx, const float* X, int64_t N, int D, con
     const int64_t count = all_pairs ? (int64_t)N * L : (int64_t)hcount;
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(&st->mode_best[0], 0, sizeof(unsigned long long) * L, s));
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(arg, 0x7f, sizeof(int32_t) * L, s));
+    // parts of a sum: enough blocks for the GPU when there are few candidates
+    int parts = 1;
+    while (!all_pairs && parts < 64 && count * parts < 8 * ctx->num_sms && count * 2 * parts <= pl.cand_cap)
+        parts *= 2;
     for (int pass = 0; pass < 2; ++pass) {
         for (int64_t c0 = 0; c0 < count; c0 += pl.cand_cap) {
             const int64_t n = std::min<int64_t>(pl.cand_cap, count - c0);
             if (pass == 0 || all_pairs) {
                 SLK_COUNT_LAUNCH(ctx, 1);
-                density_exact_kernel<<<(unsigned)n, 256, 0, s>>>(X, N, D, L, perm, off, cand,
+                density_exact_kernel<<<dim3((unsigned)n, (unsigned)parts), 256, 0, s>>>(X, N, D, L, perm, off, cand,
                                                                  all_pairs, c0, sigma_dev, fexact);
             }
             int pg = (int)((n + 255) / 256);
             if (pg > 4 * ctx->num_sms) pg = 4 * ctx->num_sms;
             SLK_COUNT_LAUNCH(ctx, 1);
-            density_pick_kernel<<<(unsigned)pg, 256, 0, s>>>(fexact, cand, c0, n, all_pairs, L, pass,
+            density_pick_kernel<<<(unsigned)pg, 256, 0, s>>>(fexact, parts, cand, c0, n, all_pairs, L, pass,
                                                              &st->mode_best[0], arg);
         }
     }

@@ -203,3 +203,17 @@ def test_kmeanspp_screened_distances(slk, N, D, L, shift, scale):
     first, u = inputs.kmeanspp_draws(N, L, seed=D)
     got = host(slk.kmeanspp(dev(X), L, first, u))
     np.testing.assert_array_equal(got, oracle.kmeanspp(X, L, first, u))
+
+
+@pytest.mark.parametrize("N,D,L,sigma", [(3000, 5, 12, 0.3), (3000, 5, 12, 3.0), (3000, 5, 12, 40.0),
+                                         (2049, 33, 40, 2.0), (4000, 2, 3, 0.05), (1500, 7, 1, 1.0)])
+def test_initial_modes_other_clusters_left_out(slk, N, D, L, sigma):
+    """Row blocks of other clusters are left out only where they cannot hold
+    the maximiser: overlapping clusters and widths from far below to far above
+    the clusters' distances, against the oracle over all pairs."""
+    X, _ = inputs.blobs(N=N, D=D, n_blobs=max(2, L // 2), centre_var=4.0, seed=N + L)
+    seeds = inputs.kmeanspp(X, L, seed=L)
+    o_modes, o_assign, o_dens = oracle.initial_modes(X, seeds, sigma)
+    g_modes, g_assign, g_dens = slk.initial_modes(dev(X), dev(seeds), sigma)
+    _check_assign(X, seeds, host(g_assign), o_assign)
+    _check_modes(X, sigma, host(g_modes), np.array(g_dens), o_modes, o_dens, o_assign)
