@@ -31,13 +31,12 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "pair32.cuh"
 #include "slk_internal.cuh"
 #include "sync.cuh"
 
 namespace {
 
-constexpr int kMsThreads = 256;
-constexpr int kMsWarps = kMsThreads / 32;
 #define kNegInf __int_as_float(0xff800000)
 
 struct MsArgs {
@@ -61,28 +60,52 @@ struct MsArgs {
     MsStatus* ms;
 };
 
-template <int R, int LG>
+template <int R, int LG, int TH>
 struct MsSmem {
-    float red[kMsWarps / (R / 4)][LG][R];  // per feature part: distances of the tile (label-major)
-    float w[R][LG];
-    float alpha[LG];
+    float red[TH / 32 / (R / 4)][LG][R];  // per feature part: distances of the tile (label-major)
+    alignas(16) float w[R][LG];
+    alignas(16) float alpha[LG];
     float mu[LG];        // running maximum of s per label
     float ssum[LG];      // running sum of weights per label (relative to mu)
     unsigned long long bar[2];
     int abort;
 };
 
-// Reduce-scatter of 64 values over the 32 lanes: afterwards lane holds the
-// full sums of original indices base, base + 1, base = 2 * bitreverse5(lane).
-__device__ __forceinline__ void reduce_scatter64(float (&v)[64], int lane) {
+// Sums of N values over the 32 lanes, scattered: halving steps while the count
+// is even (a lane keeps the half its bit selects), then whole ones.  A lane
+// ends with the sums of indices off .. off + scatter_count - 1, the same on
+// every scatter_dup lanes.
+template <int N>
+__host__ __device__ constexpr int scatter_count() {
+    int n = N;
+    for (int s = 0; s < 5; ++s)
+        if (n % 2 == 0) n /= 2;
+    return n;
+}
+template <int N>
+__host__ __device__ constexpr int scatter_dup() { return 32 * scatter_count<N>() / N; }
+template <int N>
+__device__ __forceinline__ void reduce_scatter(float (&v)[N], int lane, int& off) {
+    off = 0;
+    int n = N;
 #pragma unroll
-    for (int o = 16, n = 64; o >= 1; o >>= 1, n >>= 1) {
-        const bool up = (lane & o) != 0;
+    for (int o = 16; o >= 1; o >>= 1) {
+        if (n % 2 == 0) {
+            const bool up = (lane & o) != 0;
+            n /= 2;
 #pragma unroll
-        for (int i = 0; i < n / 2; ++i) {
-            const float keep = up ? v[i + n / 2] : v[i];
-            const float send = up ? v[i] : v[i + n / 2];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            for (int i = 0; i < N / 2; ++i) {
+                if (i < n) {
+                    const float keep = up ? v[i + n] : v[i];
+                    const float send = up ? v[i] : v[i + n];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            }
+            off += up ? n : 0;
+        } else {
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+                if (i < n) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
         }
     }
 }
@@ -90,20 +113,20 @@ __device__ __forceinline__ void reduce_scatter64(float (&v)[64], int lane) {
 // Shared-memory row stride and tile bytes.
 __host__ __device__ __forceinline__ int round4(int d) { return (d + 3) & ~3; }
 
-template <int R, int LG, int CPT>
+template <int R, int LG, int CPT, int TH>
 __device__ void ms_load_tile_plain(const MsArgs& a, float* xs, int64_t row0, int nrows) {
-    for (int i = threadIdx.x; i < R * a.Dp; i += kMsThreads) {
+    for (int i = threadIdx.x; i < R * a.Dp; i += TH) {
         const int r = i / a.Dp, c = i % a.Dp;
         xs[i] = (r < nrows && c < a.D) ? a.X[(row0 + r) * a.D + c] : 0.f;
     }
 }
 
 // Phase 1 of one unit: the weighted sums of label group g over row range pr.
-template <int R, int LG, int CPT>
+template <int R, int LG, int CPT, int TH>
 __device__ bool ms_unit(const MsArgs& a, int u, const float* Mc, float* xs0, float* xs1,
-                        float* msm, MsSmem<R, LG>& sh, uint32_t (&par)[2]) {
+                        float* msm, MsSmem<R, LG, TH>& sh, uint32_t (&par)[2]) {
     constexpr int QUADS = R / 4;
-    constexpr int HP = kMsWarps / QUADS;  // feature parts per row quad
+    constexpr int HP = TH / 32 / QUADS;   // feature parts per row quad
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int pr = u / a.groups, g = u % a.groups;
     const int l0 = g * LG;
@@ -113,20 +136,22 @@ __device__ bool ms_unit(const MsArgs& a, int u, const float* Mc, float* xs0, flo
     const float sg = *a.sigma_dev;
     const float inv2s2 = 1.0f / (2.0f * sg * sg);
 
-    // modes of the group (zero rows beyond lg)
-    for (int i = t; i < LG * Dp; i += kMsThreads) {
+    // negated modes of the group (zero rows beyond lg), two labels side by side
+    for (int i = t; i < LG * Dp; i += TH) {
         const int l = i / Dp, c = i % Dp;
-        msm[i] = (l < lg && c < D) ? __ldcg(Mc + (int64_t)(l0 + l) * D + c) : 0.f;
+        msm[((l >> 1) * Dp + c) * 2 + (l & 1)] =
+            (l < lg && c < D) ? -__ldcg(Mc + (int64_t)(l0 + l) * D + c) : 0.f;
     }
+    const pair32* m2 = reinterpret_cast<const pair32*>(msm);
     if (t < LG) {
         sh.mu[t] = kNegInf;
         sh.ssum[t] = 0.f;
     }
-    float acc[LG][CPT];
+    pair32 acc2[LG / 2][CPT];
 #pragma unroll
-    for (int l = 0; l < LG; ++l)
+    for (int l = 0; l < LG / 2; ++l)
 #pragma unroll
-        for (int c = 0; c < CPT; ++c) acc[l][c] = 0.f;
+        for (int c = 0; c < CPT; ++c) acc2[l][c] = pack2(0.f, 0.f);
     __syncthreads();
 
     auto issue = [&](int64_t ti, int b) {
@@ -141,7 +166,7 @@ __device__ bool ms_unit(const MsArgs& a, int u, const float* Mc, float* xs0, flo
                 bulk_g2s(dst, a.X + row0 * D, bytes, &sh.bar[b]);
             }
         } else {
-            ms_load_tile_plain<R, LG, CPT>(a, dst, row0, nrows);
+            ms_load_tile_plain<R, LG, CPT, TH>(a, dst, row0, nrows);
         }
     };
 
@@ -163,58 +188,79 @@ __device__ bool ms_unit(const MsArgs& a, int u, const float* Mc, float* xs0, flo
             __syncthreads();
         }
 
+        // phase B's log z, loaded ahead of the distances: R lanes per label,
+        // lane = row
+        constexpr int BL = 32 / R, BP = (LG + BL * (TH / 32) - 1) / (BL * (TH / 32));
+        const int brow = lane % R;
+        float lz[BP];
+#pragma unroll
+        for (int q = 0; q < BP; ++q) {
+            const int l = (q * (TH / 32) + warp) * BL + lane / R;
+            lz[q] = (l < lg && brow < nrows) ? __ldg(a.LZ + (row0 + brow) * a.L + l0 + l) : 0.f;
+        }
         // ---- A: distances of 4 rows x LG labels over a part of the features
         {
             const int q = warp % QUADS, h = warp / QUADS;
-            float v[64];
+            pair32 v2[4][LG / 2];
 #pragma unroll
-            for (int i = 0; i < 64; ++i) v[i] = 0.f;
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int l = 0; l < LG / 2; ++l) v2[i][l] = pack2(0.f, 0.f);
             const float* x0 = xs + (4 * q) * Dp;
             for (int c0 = h * 32; c0 < D; c0 += HP * 32) {
                 const int d = c0 + lane;
                 if (d < D) {
-                    const float x[4] = {x0[d], x0[Dp + d], x0[2 * Dp + d], x0[3 * Dp + d]};
+                    const pair32 x[4] = {pack2(x0[d], x0[d]), pack2(x0[Dp + d], x0[Dp + d]),
+                                         pack2(x0[2 * Dp + d], x0[2 * Dp + d]),
+                                         pack2(x0[3 * Dp + d], x0[3 * Dp + d])};
 #pragma unroll
-                    for (int l = 0; l < LG; ++l) {
-                        const float m = msm[l * Dp + d];
+                    for (int l = 0; l < LG / 2; ++l) {
+                        const pair32 m = m2[l * Dp + d];
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            const float df = x[i] - m;
-                            v[i * 16 + l] = fmaf(df, df, v[i * 16 + l]);
+                            const pair32 df = add2(x[i], m);
+                            v2[i][l] = fma2(df, df, v2[i][l]);
                         }
                     }
                 }
             }
-            reduce_scatter64(v, lane);
-            const int base = (((lane >> 4) & 1) << 5) | (((lane >> 3) & 1) << 4) |
-                             (((lane >> 2) & 1) << 3) | (((lane >> 1) & 1) << 2) | ((lane & 1) << 1);
-            const int i = base >> 4, l = base & 15;
-            if (l < LG) sh.red[h][l][4 * q + i] = v[0];
-            if (l + 1 < LG) sh.red[h][l + 1][4 * q + i] = v[1];
+            float v[4 * LG];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int l = 0; l < LG / 2; ++l) unpack2(v2[i][l], v[i * LG + 2 * l], v[i * LG + 2 * l + 1]);
+            int off;
+            reduce_scatter<4 * LG>(v, lane, off);
+            if (lane % scatter_dup<4 * LG>() == 0)
+#pragma unroll
+            for (int i = 0; i < scatter_count<4 * LG>(); ++i)
+                sh.red[h][(off + i) % LG][4 * q + (off + i) / LG] = v[i];
         }
         __syncthreads();
-        // ---- B: a warp per label (labels warp, warp + 8, ...), lanes over the
-        // rows: s, tile maximum, rescale factor of the running sums, weights
-        // relative to the new maximum
-        for (int l = warp; l < LG; l += kMsWarps) {
+        // ---- B: R lanes per label, lane = row: s, tile maximum, rescale factor
+        // of the running sums, weights relative to the new maximum
+#pragma unroll
+        for (int q = 0; q < BP; ++q) {
+            const int l = (q * (TH / 32) + warp) * BL + lane / R;
+            const bool on = l < LG;
             float sv = kNegInf;
-            if (lane < R && lane < nrows && l < lg) {
+            if (brow < nrows && l < lg) {
                 float d2 = 0.f;
 #pragma unroll
-                for (int hh = 0; hh < HP; ++hh) d2 += sh.red[hh][l][lane];
-                sv = __ldg(a.LZ + (row0 + lane) * a.L + l0 + l) - d2 * inv2s2;
+                for (int hh = 0; hh < HP; ++hh) d2 += sh.red[hh][l][brow];
+                sv = lz[q] - d2 * inv2s2;
             }
             float tm = sv;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) tm = fmaxf(tm, __shfl_xor_sync(0xffffffffu, tm, o));
-            const float mo = sh.mu[l];
+            for (int o = R / 2; o > 0; o >>= 1) tm = fmaxf(tm, __shfl_xor_sync(0xffffffffu, tm, o));
+            const float mo = on ? sh.mu[l] : kNegInf;
             const float mn = fmaxf(mo, tm);
             const float wt = (sv == kNegInf) ? 0.f : expf(sv - mn);
-            if (lane < R) sh.w[lane][l] = wt;
+            if (on) sh.w[brow][l] = wt;
             float sw = wt;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sw += __shfl_xor_sync(0xffffffffu, sw, o);
-            if (lane == 0) {
+            for (int o = R / 2; o > 0; o >>= 1) sw += __shfl_xor_sync(0xffffffffu, sw, o);
+            if (on && brow == 0) {
                 const float al = (mn == kNegInf) ? 1.f : expf(mo - mn);
                 sh.alpha[l] = al;
                 sh.mu[l] = mn;
@@ -224,26 +270,25 @@ __device__ bool ms_unit(const MsArgs& a, int u, const float* Mc, float* xs0, flo
         __syncthreads();
         // ---- C: rescale and accumulate the weighted rows
         {
-            float al[LG];
+            const pair32* al = reinterpret_cast<const pair32*>(sh.alpha);
 #pragma unroll
-            for (int l = 0; l < LG; ++l) al[l] = sh.alpha[l];
+            for (int l = 0; l < LG / 2; ++l)
 #pragma unroll
-            for (int l = 0; l < LG; ++l)
-#pragma unroll
-                for (int c = 0; c < CPT; ++c) acc[l][c] *= al[l];
+                for (int c = 0; c < CPT; ++c) acc2[l][c] = mul2(acc2[l][c], al[l]);
             for (int r = 0; r < nrows; ++r) {
-                float wv[LG];
+                pair32 wv[LG / 2];
 #pragma unroll
                 for (int l = 0; l < LG; l += 4) {
-                    const float4 w4 = *reinterpret_cast<const float4*>(&sh.w[r][l]);
-                    wv[l] = w4.x; wv[l + 1] = w4.y; wv[l + 2] = w4.z; wv[l + 3] = w4.w;
+                    const ulonglong2 w4 = *reinterpret_cast<const ulonglong2*>(&sh.w[r][l]);
+                    wv[l / 2] = w4.x;
+                    wv[l / 2 + 1] = w4.y;
                 }
                 const float* xr = xs + r * Dp;
                 float xv[CPT];
                 if constexpr (CPT >= 4) {
 #pragma unroll
                     for (int j = 0; j < CPT / 4; ++j) {
-                        const int q4 = t + kMsThreads * j;
+                        const int q4 = t + TH * j;
                         float4 x4 = make_float4(0.f, 0.f, 0.f, 0.f);
                         if (4 * q4 < Dp) x4 = *reinterpret_cast<const float4*>(xr + 4 * q4);
                         xv[4 * j] = x4.x; xv[4 * j + 1] = x4.y; xv[4 * j + 2] = x4.z; xv[4 * j + 3] = x4.w;
@@ -261,15 +306,22 @@ __device__ bool ms_unit(const MsArgs& a, int u, const float* Mc, float* xs0, flo
                     }
                 }
 #pragma unroll
-                for (int l = 0; l < LG; ++l)
+                for (int c = 0; c < CPT; ++c) {
+                    const pair32 x2 = pack2(xv[c], xv[c]);
 #pragma unroll
-                    for (int c = 0; c < CPT; ++c) acc[l][c] = fmaf(wv[l], xv[c], acc[l][c]);
+                    for (int l = 0; l < LG / 2; ++l) acc2[l][c] = fma2(wv[l], x2, acc2[l][c]);
+                }
             }
         }
         __syncthreads();  // the buffer and the tile's weights are free again
     }
 
     // unit results
+    float acc[LG][CPT];
+#pragma unroll
+    for (int l = 0; l < LG / 2; ++l)
+#pragma unroll
+        for (int c = 0; c < CPT; ++c) unpack2(acc2[l][c], acc[2 * l][c], acc[2 * l + 1][c]);
     float* pu = a.part + (int64_t)u * LG * D;
 #pragma unroll
     for (int l = 0; l < LG; ++l) {
@@ -277,7 +329,7 @@ __device__ bool ms_unit(const MsArgs& a, int u, const float* Mc, float* xs0, flo
         if constexpr (CPT >= 4) {
 #pragma unroll
             for (int j = 0; j < CPT / 4; ++j) {
-                const int q4 = t + kMsThreads * j;
+                const int q4 = t + TH * j;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     const int col = 4 * q4 + c;
@@ -300,13 +352,16 @@ __device__ bool ms_unit(const MsArgs& a, int u, const float* Mc, float* xs0, flo
     return true;
 }
 
-// Phase 2: warps over (label, 32 features): combine the units of the
-// label's group in float64, new mode, squared move added per label.
-template <int LG>
+// Phase 2: warps over (label, 32 features): combine the units of the label's
+// group in float64, new mode, squared move added per label.  The units come 32
+// at a time: lane = unit for the scale factors, lane = feature for the sums,
+// whose loads then do not wait on one another.
+template <int LG, int TH>
 __device__ void ms_finish(const MsArgs& a, int it, float* Mnext) {
     const int lane = threadIdx.x & 31;
-    const int64_t gw = (int64_t)blockIdx.x * kMsWarps + (threadIdx.x >> 5);
-    const int64_t nw = (int64_t)gridDim.x * kMsWarps;
+    // neighbouring tasks on different SMs (an SM runs 2 float64 lanes a clock)
+    const int64_t gw = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const int64_t nw = (int64_t)gridDim.x * (TH / 32);
     const int D = a.D;
     const int nblk = (D + 31) / 32;
     double* sh2 = a.ms->shift2[it % 3];
@@ -315,15 +370,32 @@ __device__ void ms_finish(const MsArgs& a, int it, float* Mnext) {
         const int d = (int)(task % nblk) * 32 + lane;
         const int g = l / LG, li = l % LG;
         float mu = kNegInf;
-        for (int p = 0; p < a.P; ++p) mu = fmaxf(mu, __ldcg(a.part_mu + (p * a.groups + g) * LG + li));
+        for (int p = lane; p < a.P; p += 32) mu = fmaxf(mu, __ldcg(a.part_mu + (p * a.groups + g) * LG + li));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mu = fmaxf(mu, __shfl_xor_sync(0xffffffffu, mu, o));
         double num = 0.0, den = 0.0;
-        for (int p = 0; p < a.P; ++p) {
-            const int uu = p * a.groups + g;
-            const float mp = __ldcg(a.part_mu + uu * LG + li);
-            const double c = (mp == kNegInf) ? 0.0 : (double)expf(mp - mu);
-            den += c * (double)__ldcg(a.part_s + uu * LG + li);
-            if (d < D) num += c * (double)__ldcg(a.part + ((int64_t)uu * LG + li) * D + d);
+        for (int p0 = 0; p0 < a.P; p0 += 32) {
+            const int n = min(32, a.P - p0);
+            double c = 0.0;
+            if (lane < n) {
+                const int uu = (p0 + lane) * a.groups + g;
+                const float mp = __ldcg(a.part_mu + uu * LG + li);
+                c = (mp == kNegInf) ? 0.0 : (double)expf(mp - mu);
+                den += c * (double)__ldcg(a.part_s + uu * LG + li);
+            }
+            const float* src = a.part + ((int64_t)(p0 * a.groups + g) * LG + li) * D + d;
+            const int64_t step = (int64_t)a.groups * LG * D;
+            for (int q0 = 0; q0 < n; q0 += 8) {
+                float v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) v[q] = (q0 + q < n && d < D) ? __ldcg(src + (q0 + q) * step) : 0.f;
+#pragma unroll
+                for (int q = 0; q < 8; ++q)   // c is 0 beyond n (q0 + q < 32)
+                    num += __shfl_sync(0xffffffffu, c, q0 + q) * (double)v[q];
+            }
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
         double mv = 0.0;
         if (d < D) {
             const int64_t o = (int64_t)l * D + d;
@@ -351,30 +423,30 @@ __device__ __forceinline__ bool ms_decide(const MsArgs& a, int it) {
     return a.tol >= 0.f && shift <= a.tol * *a.sigma_dev;
 }
 
-template <int R, int LG, int CPT>
+template <int R, int LG, int CPT, int TH>
 struct MsLayout {
     static size_t bytes(int Dp) {
-        return 1024 + sizeof(MsSmem<R, LG>) + sizeof(float) * ((size_t)2 * R * Dp + (size_t)LG * Dp);
+        return 1024 + sizeof(MsSmem<R, LG, TH>) + sizeof(float) * ((size_t)2 * R * Dp + (size_t)LG * Dp);
     }
 };
 
-template <int R, int LG, int CPT>
-__device__ __forceinline__ void ms_carve(unsigned char* raw, int Dp, MsSmem<R, LG>*& sh,
+template <int R, int LG, int CPT, int TH>
+__device__ __forceinline__ void ms_carve(unsigned char* raw, int Dp, MsSmem<R, LG, TH>*& sh,
                                          float*& xs0, float*& xs1, float*& msm) {
     unsigned char* base =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(raw) + 127) & ~uintptr_t(127));
     xs0 = reinterpret_cast<float*>(base);
     xs1 = xs0 + (size_t)R * Dp;
     msm = xs1 + (size_t)R * Dp;
-    sh = reinterpret_cast<MsSmem<R, LG>*>(msm + (size_t)LG * Dp);
+    sh = reinterpret_cast<MsSmem<R, LG, TH>*>(msm + (size_t)LG * Dp);
 }
 
-template <int R, int LG, int CPT>
-__global__ void __launch_bounds__(kMsThreads, 1) ms_persistent_kernel(MsArgs a) {
+template <int R, int LG, int CPT, int TH>
+__global__ void __launch_bounds__(TH, 1) ms_persistent_kernel(MsArgs a) {
     extern __shared__ unsigned char ms_raw[];
-    MsSmem<R, LG>* sh;
+    MsSmem<R, LG, TH>* sh;
     float *xs0, *xs1, *msm;
-    ms_carve<R, LG, CPT>(ms_raw, a.Dp, sh, xs0, xs1, msm);
+    ms_carve<R, LG, CPT, TH>(ms_raw, a.Dp, sh, xs0, xs1, msm);
     GridBarrier* gb = reinterpret_cast<GridBarrier*>(a.ms);
     if (threadIdx.x == 0) {
         mbar_init1(&sh->bar[0]);
@@ -387,15 +459,15 @@ __global__ void __launch_bounds__(kMsThreads, 1) ms_persistent_kernel(MsArgs a) 
     for (int it = 0; it < a.max_iters; ++it) {
         const float* Mc = (it == 0) ? a.Mout : a.Mbuf[(it - 1) & 1];
         if (blockIdx.x == 0)
-            for (int l = threadIdx.x; l < a.L; l += kMsThreads) a.ms->shift2[(it + 1) % 3][l] = 0.0;
+            for (int l = threadIdx.x; l < a.L; l += TH) a.ms->shift2[(it + 1) % 3][l] = 0.0;
         for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x)
-            ok = ms_unit<R, LG, CPT>(a, u, Mc, xs0, xs1, msm, *sh, par);
+            ok = ms_unit<R, LG, CPT, TH>(a, u, Mc, xs0, xs1, msm, *sh, par);
         if (!ok) {
             if (threadIdx.x == 0) atomicOr(&gb->error, 2u);
             break;
         }
         if (grid_barrier(gb, gridDim.x, [] { return false; }) < 0) break;
-        ms_finish<LG>(a, it, a.Mbuf[it & 1]);
+        ms_finish<LG, TH>(a, it, a.Mbuf[it & 1]);
         const int r = grid_barrier(gb, gridDim.x, [&] { return ms_decide(a, it); });
         if (r != 0) break;
     }
@@ -412,13 +484,13 @@ __global__ void __launch_bounds__(kMsThreads, 1) ms_persistent_kernel(MsArgs a) 
 
 // Without cooperative launch: one launch per phase and iteration; a launch
 // after the decision has stopped the loop returns at once.
-template <int R, int LG, int CPT>
-__global__ void __launch_bounds__(kMsThreads, 1) ms_accum_kernel(MsArgs a, int it) {
+template <int R, int LG, int CPT, int TH>
+__global__ void __launch_bounds__(TH, 1) ms_accum_kernel(MsArgs a, int it) {
     if (*(volatile unsigned*)&a.ms->stop != 0u) return;
     extern __shared__ unsigned char ms_raw[];
-    MsSmem<R, LG>* sh;
+    MsSmem<R, LG, TH>* sh;
     float *xs0, *xs1, *msm;
-    ms_carve<R, LG, CPT>(ms_raw, a.Dp, sh, xs0, xs1, msm);
+    ms_carve<R, LG, CPT, TH>(ms_raw, a.Dp, sh, xs0, xs1, msm);
     if (threadIdx.x == 0) {
         mbar_init1(&sh->bar[0]);
         mbar_init1(&sh->bar[1]);
@@ -427,11 +499,11 @@ __global__ void __launch_bounds__(kMsThreads, 1) ms_accum_kernel(MsArgs a, int i
     __syncthreads();
     const float* Mc = (it == 0) ? a.Mout : a.Mbuf[(it - 1) & 1];
     if (blockIdx.x == 0)
-        for (int l = threadIdx.x; l < a.L; l += kMsThreads) a.ms->shift2[(it + 1) % 3][l] = 0.0;
+        for (int l = threadIdx.x; l < a.L; l += TH) a.ms->shift2[(it + 1) % 3][l] = 0.0;
     uint32_t par[2] = {0u, 0u};
     bool ok = true;
     for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x)
-        ok = ms_unit<R, LG, CPT>(a, u, Mc, xs0, xs1, msm, *sh, par);
+        ok = ms_unit<R, LG, CPT, TH>(a, u, Mc, xs0, xs1, msm, *sh, par);
     if (!ok && threadIdx.x == 0) {
         atomicOr(&a.ms->error, 2u);
         for (int b = 0; b < 2; ++b) mbar_wait_parity(&sh->bar[b], par[b]);
@@ -443,10 +515,10 @@ __global__ void __launch_bounds__(kMsThreads, 1) ms_accum_kernel(MsArgs a, int i
     }
 }
 
-template <int LG>
-__global__ void __launch_bounds__(kMsThreads) ms_finish_kernel(MsArgs a, int it) {
+template <int LG, int TH>
+__global__ void __launch_bounds__(TH) ms_finish_kernel(MsArgs a, int it) {
     if (*(volatile unsigned*)&a.ms->stop != 0u || *(volatile unsigned*)&a.ms->error != 0u) return;
-    ms_finish<LG>(a, it, a.Mbuf[it & 1]);
+    ms_finish<LG, TH>(a, it, a.Mbuf[it & 1]);
     __shared__ int last;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -514,29 +586,33 @@ ms_moved_kernel(const double* __restrict__ M64, const double* __restrict__ M0, i
 }
 
 // Launch shape for a feature count: rows per tile, labels per group,
-// features per thread in phase C.
+// features per thread in phase C, threads.  Up to 1024 features 512 threads:
+// the tile's phases are chains of shared-memory loads and shuffles between
+// barriers, and 8 warps (2 per scheduler) leave the float32 units idle four
+// fifths of the time (70000 x 784, L = 10: MS_FIGURES); beyond, the
+// accumulators of a thread and the rows' shared memory leave room for 256.
 struct MsShape {
-    int R, LG, CPT;
+    int R, LG, CPT, TH;
 };
 MsShape ms_shape(int D, int L) {
     if (D <= 1024) {
-        const int cpt = D <= 256 ? 1 : D <= 512 ? 2 : 4;
+        const int cpt = D <= 512 ? 1 : 2;
         const int lg = L <= 4 ? 4 : L <= 8 ? 8 : L <= 12 ? 12 : 16;
-        return {16, lg, cpt};
+        return {16, lg, cpt, 512};
     }
-    if (D <= 2048) return {8, L <= 4 ? 4 : 8, 8};
-    return {4, 4, 16};
+    if (D <= 2048) return {8, L <= 4 ? 4 : 8, 8, 256};
+    return {4, 4, 16, 256};
 }
 
-template <int R, int LG, int CPT>
+template <int R, int LG, int CPT, int TH>
 slk_status ms_run(slk_ctx* ctx, MsArgs& a) {
-    const size_t smem = MsLayout<R, LG, CPT>::bytes(a.Dp);
-    auto kp = ms_persistent_kernel<R, LG, CPT>;
-    auto ka = ms_accum_kernel<R, LG, CPT>;
+    const size_t smem = MsLayout<R, LG, CPT, TH>::bytes(a.Dp);
+    auto kp = ms_persistent_kernel<R, LG, CPT, TH>;
+    auto ka = ms_accum_kernel<R, LG, CPT, TH>;
     SLK_CUDA_TRY(ctx, cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     SLK_CUDA_TRY(ctx, cudaFuncSetAttribute(ka, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    SLK_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kp, kMsThreads, smem));
+    SLK_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kp, TH, smem));
     if (per_sm < 1) return set_err(ctx, SLK_ERR_CUDA, "mean-shift kernel does not fit on an SM");
     // the workspace holds the partial sums of at most 2 CTAs per SM
     const int64_t max_grid = (int64_t)ctx->num_sms * (per_sm < 2 ? per_sm : 2);
@@ -550,13 +626,13 @@ slk_status ms_run(slk_ctx* ctx, MsArgs& a) {
         SLK_COUNT_LAUNCH(ctx, 1);
         void* args[] = {&a};
         cudaError_t e = cudaLaunchCooperativeKernel((const void*)kp, dim3((unsigned)grid),
-                                                    dim3(kMsThreads), args, smem, ctx->stream);
+                                                    dim3(TH), args, smem, ctx->stream);
         if (e != cudaSuccess) return cuda_err(ctx, e, "ms_persistent_kernel");
     } else {
         SLK_COUNT_LAUNCH(ctx, 2 * a.max_iters);
         for (int it = 0; it < a.max_iters; ++it) {
-            ka<<<(unsigned)grid, kMsThreads, smem, ctx->stream>>>(a, it);
-            ms_finish_kernel<LG><<<(unsigned)grid, kMsThreads, 0, ctx->stream>>>(a, it);
+            ka<<<(unsigned)grid, TH, smem, ctx->stream>>>(a, it);
+            ms_finish_kernel<LG, TH><<<(unsigned)grid, TH, 0, ctx->stream>>>(a, it);
         }
         SLK_LAUNCH_CHECK(ctx, "ms_accum_kernel / ms_finish_kernel");
     }
@@ -604,13 +680,12 @@ slk_status ms_launch(slk_ctx* ctx, const float* X, int64_t N, int D, const float
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(ms, 0, sizeof(MsStatus), ctx->stream));
     if (max_iters <= 0) return SLK_OK;
     PhaseScope ps(ctx, SLK_PHASE_MEANSHIFT);
-#define SLK_MS(R_, LG_, CPT_) \
-    if (s.R == R_ && s.LG == LG_ && s.CPT == CPT_) return ms_run<R_, LG_, CPT_>(ctx, a);
-    SLK_MS(16, 4, 1) SLK_MS(16, 8, 1) SLK_MS(16, 12, 1) SLK_MS(16, 16, 1)
-    SLK_MS(16, 4, 2) SLK_MS(16, 8, 2) SLK_MS(16, 12, 2) SLK_MS(16, 16, 2)
-    SLK_MS(16, 4, 4) SLK_MS(16, 8, 4) SLK_MS(16, 12, 4) SLK_MS(16, 16, 4)
-    SLK_MS(8, 4, 8) SLK_MS(8, 8, 8)
-    SLK_MS(4, 4, 16)
+#define SLK_MS(R_, LG_, CPT_, TH_) \
+    if (s.R == R_ && s.LG == LG_ && s.CPT == CPT_) return ms_run<R_, LG_, CPT_, TH_>(ctx, a);
+    SLK_MS(16, 4, 1, 512) SLK_MS(16, 8, 1, 512) SLK_MS(16, 12, 1, 512) SLK_MS(16, 16, 1, 512)
+    SLK_MS(16, 4, 2, 512) SLK_MS(16, 8, 2, 512) SLK_MS(16, 12, 2, 512) SLK_MS(16, 16, 2, 512)
+    SLK_MS(8, 4, 8, 256) SLK_MS(8, 8, 8, 256)
+    SLK_MS(4, 4, 16, 256)
 #undef SLK_MS
     return set_err(ctx, SLK_ERR_INVALID_ARG, "mean-shift modes: no launch shape");
 }
