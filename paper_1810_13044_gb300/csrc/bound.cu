@@ -353,6 +353,185 @@ bound_persistent_kernel(const float* __restrict__ A, const int64_t* __restrict__
     if (blockIdx.x == 0 && threadIdx.x == 0) st->iters_done = it;
 }
 
+// One row of cnt edges from e0, windows of W neighbours; q and wq hold the names
+// and weights of the first NP G edges (edge G i + lane in place i), those of the
+// next windows arrive while one is summed.  The arithmetic of rows_update, bit
+// for bit.
+template <int G, int LPL, int W>
+__device__ __forceinline__ float row_update_named(int64_t p, int64_t e0, int cnt, int (&q)[(W + G - 1) / G],
+                                                  float (&wq)[(W + G - 1) / G], int gl, unsigned gmask,
+                                                  const float* __restrict__ A,
+                                                  const int32_t* __restrict__ col_idx,
+                                                  const float* __restrict__ w, const float* Zin, float* Zout,
+                                                  int L, float lambda) {
+    constexpr int NP = (W + G - 1) / G;
+    constexpr int STEP = W < G ? G : W;   // edges whose names are held
+    float av[LPL], zo[LPL], b[LPL];
+#pragma unroll
+    for (int j = 0; j < LPL; ++j) {
+        const int l = gl + G * j;
+        av[j] = l < L ? __ldg(A + p * (int64_t)L + l) : 0.f;
+        zo[j] = l < L ? __ldcg(Zin + p * (int64_t)L + l) : 0.f;
+        b[j] = 0.f;
+    }
+    for (int c0 = 0; c0 < cnt; c0 += STEP) {
+        int qn[NP];
+        float wn[NP];
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            const int e = c0 + STEP + G * i + gl;
+            qn[i] = e < cnt ? __ldg(col_idx + e0 + e) : 0;
+            wn[i] = e < cnt && w ? __ldg(w + e0 + e) : 1.f;
+        }
+#pragma unroll
+        for (int t0 = 0; t0 < STEP; t0 += W) {
+            if (c0 + t0 >= cnt) break;   // uniform within the group
+            float zz[W][LPL], ww[W];
+#pragma unroll
+            for (int u = 0; u < W; ++u) {
+                const int qu = __shfl_sync(gmask, q[(t0 + u) / G], (t0 + u) % G, G);
+                ww[u] = __shfl_sync(gmask, wq[(t0 + u) / G], (t0 + u) % G, G);
+                const float* zq = Zin + (int64_t)qu * L;
+#pragma unroll
+                for (int j = 0; j < LPL; ++j) {
+                    const int l = gl + G * j;
+                    zz[u][j] = (c0 + t0 + u < cnt && l < L) ? __ldcg(zq + l) : 0.f;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < W; ++u)
+                if (c0 + t0 + u < cnt)
+#pragma unroll
+                    for (int j = 0; j < LPL; ++j) b[j] = fmaf(ww[u], zz[u][j], b[j]);
+        }
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            q[i] = qn[i];
+            wq[i] = wn[i];
+        }
+    }
+    float sv[LPL], m = -INFINITY;
+#pragma unroll
+    for (int j = 0; j < LPL; ++j) {
+        sv[j] = gl + G * j < L ? fmaf(lambda, b[j], av[j]) : -INFINITY;
+        m = fmaxf(m, sv[j]);
+    }
+    m = group_max<G>(m, gmask);
+    float e[LPL], sum = 0.f, d = 0.f;
+#pragma unroll
+    for (int j = 0; j < LPL; ++j) {
+        e[j] = (gl + G * j < L) ? expf(sv[j] - m) : 0.f;
+        sum += e[j];
+    }
+    sum = group_sum<G>(sum, gmask);
+#pragma unroll
+    for (int j = 0; j < LPL; ++j) {
+        const int l = gl + G * j;
+        if (l < L) {
+            const float z = e[j] / sum;
+            d = fmaxf(d, fabsf(z - zo[j]));
+            __stcg(Zout + p * (int64_t)L + l, z);
+        }
+    }
+    return d;
+}
+
+// Persistent inner loop over rows of any degree (the symmetric affinity).  Bound
+// by the latency of gathering neighbours and by the slowest group before the
+// grid's barrier, not by bandwidth (L2 at a fifth): so a block's rows are a
+// queue its lane groups take from, hubs (more than kHubDeg edges, listed once
+// per launch) first, and a group has up to 16 neighbours' labels under way
+// while the next row's names and the offsets of the one after arrive.
+// Measured on the symmetric graph of 60001 x 50 points, k = 8 (mean degree
+// 13.6, largest 409), L = 30, 100 updates: 10.8 ms with every group on a fixed
+// set of rows and a neighbour's load waiting for its name; 8.1 with names
+// ahead and hubs first, windows of 8, three blocks per SM; 7.3 with the queue;
+// 5.9 with windows of 16 and two blocks per SM (32: 6.4; four blocks: 7.3).
+constexpr int kHubDeg = 48, kHubMax = 512;
+template <int G, int LPL>
+__global__ void __launch_bounds__(kThreads, 2)
+bound_var_kernel(const float* __restrict__ A, const int64_t* __restrict__ row_ptr,
+                 const int32_t* __restrict__ col_idx, const float* __restrict__ w,
+                 int64_t N, int L, float lambda, float* Z0, float* Z1, int max_iters,
+                 float tol, DevState* st) {
+    constexpr int RPW = 32 / G, W = LPL > 2 ? 32 / LPL : G < 16 ? G : 16;   // neighbours in flight
+    __shared__ float red[kThreads / 32];
+    __shared__ int hub[kHubMax], n_hub, next[2];
+    const int lane = threadIdx.x & 31;
+    const int gl = lane % G, grp = lane / G;
+    const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (grp * G));
+    constexpr int PER = (kThreads / 32) * RPW;   // groups of a block
+    // item k of the block: its hubs, then PER consecutive rows of every grid stride
+    const int64_t stride = (int64_t)gridDim.x * PER, first = (int64_t)blockIdx.x * PER;
+    if (threadIdx.x == 0) n_hub = next[0] = next[1] = 0;
+    __syncthreads();
+    for (int64_t k = threadIdx.x;; k += kThreads) {
+        const int64_t p = first + (k / PER) * stride + k % PER;
+        if (first + (k / PER) * stride >= N) break;
+        if (p < N && __ldg(row_ptr + p + 1) - __ldg(row_ptr + p) > kHubDeg) {
+            const int at = atomicAdd(&n_hub, 1);
+            if (at < kHubMax) hub[at] = (int)p;
+        }
+    }
+    __syncthreads();
+    // more than fit: every row stays where it is
+    const int hubs = n_hub <= kHubMax ? n_hub : 0, maxdeg = n_hub <= kHubMax ? kHubDeg : 0x7fffffff;
+    auto names = [&](int64_t e, int c, int& q, float& x) {
+        q = gl < c ? __ldg(col_idx + e + gl) : 0;
+        x = gl < c && w ? __ldg(w + e + gl) : 1.f;
+    };
+    int it = 0;
+    while (it < max_iters) {
+        const float* Zin = (it & 1) ? Z1 : Z0;
+        float* Zout = (it & 1) ? Z0 : Z1;
+        float d = 0.f;
+        // the group's next item, its row, offset and degree (-1: a hub, done before)
+        auto take = [&](int64_t& p, int64_t& e, int& c) {
+            int k = 0;
+            if (gl == 0) k = atomicAdd(&next[it & 1], 1);
+            k = __shfl_sync(gmask, k, 0, G);
+            e = 0;
+            c = -1;
+            p = k < hubs ? hub[k] : first + (int64_t)((k - hubs) / PER) * stride + (k - hubs) % PER;
+            if (p >= N) {
+                if (p - (k - hubs) % PER >= N) p = -1;   // no more rows
+                return;
+            }
+            e = __ldg(row_ptr + p);
+            c = (int)(__ldg(row_ptr + p + 1) - e);
+            if (k >= hubs && c > maxdeg) c = -1;
+        };
+        int64_t p1, p2, e1, e2;
+        int c1, c2, q1;
+        float x1;
+        take(p1, e1, c1);
+        names(e1, c1, q1, x1);
+        take(p2, e2, c2);
+        while (p1 >= 0) {
+            const int64_t p = p1, e = e1;
+            const int c = c1;
+            int q[1] = {q1};
+            float x[1] = {x1};
+            p1 = p2;
+            e1 = e2;
+            c1 = c2;
+            names(e1, c1, q1, x1);
+            if (p1 >= 0) take(p2, e2, c2);
+            if (c >= 0)   // uniform within the group
+                d = fmaxf(d, row_update_named<G, LPL, W>(p, e, c, q, x, gl, gmask, A, col_idx, w, Zin, Zout, L,
+                                                         lambda));
+        }
+        if (threadIdx.x == 0) next[(it + 1) & 1] = 0;   // last read before the last step's barrier
+        const float bm = block_max(d, red);
+        if (threadIdx.x == 0) atomicMax(&st->delta_bits[it % 3], __float_as_uint(bm));
+        const int r = grid_step(st, gridDim.x, it, tol);
+        if (r < 0) return;
+        ++it;
+        if (r == 1) break;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->iters_done = it;
+}
+
 // ------------------------------------------------ 16-byte form for 64 < L <= 128
 //
 // For L a multiple of 4 in (64, 128] one warp owns a row and lane v owns the
@@ -1211,6 +1390,25 @@ slk_status bound_launch(slk_ctx* ctx, const float* A, const int64_t* row_ptr,
             if (e != cudaSuccess) return cuda_err(ctx, e, "bound_vec4_kernel");
             cached = true;   // launched: skip the label-strided kernel below
         }
+#define SLK_LAUNCH_VAR(G_, LPL_)                                                               \
+    if (!cached && kdeg == 0) {                                                                \
+        auto kern = bound_var_kernel<G_, LPL_>;                                                \
+        int per_sm = 0;                                                                        \
+        SLK_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, 0)); \
+        if (per_sm < 1) return set_err(ctx, SLK_ERR_CUDA, "bound kernel cannot be resident"); \
+        int64_t grid = (int64_t)per_sm * ctx->num_sms;                                         \
+        if (grid > blocks_needed) grid = blocks_needed;                                        \
+        const float* a_ = A; const int64_t* rp_ = row_ptr; const int32_t* ci_ = col_idx;       \
+        const float* w_ = w; int64_t n_ = N; int l_ = L; float lam_ = lambda;                  \
+        float* z0_ = Z; float* z1_ = Z_prev; int mi_ = max_iters; float tol_ = tol;            \
+        DevState* st_ = st;                                                                    \
+        void* args[] = {&a_, &rp_, &ci_, &w_, &n_, &l_, &lam_, &z0_, &z1_, &mi_, &tol_, &st_}; \
+        e = cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)grid), dim3(kThreads), \
+                                        args, 0, ctx->stream);                                 \
+        cached = true;                                                                         \
+    }
+        SLK_DISPATCH_L(L, SLK_LAUNCH_VAR);
+#undef SLK_LAUNCH_VAR
 #define SLK_LAUNCH_PERSISTENT(G_, LPL_)                                                        \
     if (!cached) {                                                                             \
         auto kern = bound_persistent_kernel<G_, LPL_>;                                         \
