@@ -15,7 +15,8 @@
 //   sym_rows_kernel<1>    per row: merge into K' (deterministic: both lists
 //                         sorted), weights 0.5 (w_pq + w_qp)
 // One thread per row; in-lists are short except at hubs, whose insertion sort
-// by one thread was the cost (60001 x 50, k = 8, hubs of 1000: SYM_FIGURES).
+// by one thread was the cost (60001 x 50, k = 8, in-lists up to 409: sym_rows_kernel<0>
+// 2.44 ms; with the long lists ranked before it 0.10 + 0.14 ms).
 #include <stdint.h>
 
 #include "slk_internal.cuh"
