@@ -32,12 +32,12 @@
 #include "knn_cert.cuh"
 #include "knn_group.cuh"
 #include "knn_sweep.cuh"
+#include "pair32.cuh"
 #include "slk_internal.cuh"
 
 namespace {
 
 constexpr int BM = 128, BN = 128, BK = 16, KT = 256;
-constexpr int QC = 32;      // per-row insertion queue of the candidate kernel
 constexpr int MAXE = 16;    // merge entries per lane (splits * KC <= 512)
 #define kInf __int_as_float(0x7f800000)
 constexpr int kNoIdx = 0x7fffffff;
@@ -160,6 +160,10 @@ __device__ __forceinline__ void rho_kappa(float eh, float el, float vh, float vl
     kappa = (v2 > 0.f) ? (vlo > 0.f ? __fdiv_ru(rho, vlo) : __int_as_float(0x7f800000)) : 0.f;
 }
 
+// Form of the candidate operand: bfloat16 or float32 rows, or float32 tiles of
+// 128 rows by feature ([Np / 128][Dp][128]), as the float32 kernel stages them.
+enum class Operand { bf16, f32_rows, f32_tiles };
+
 // One warp per padded row: xt = round(v), v = fl(x - mu), with
 //   norms[p] = ||xt_p||^2: lane sums of xt^2 in float32, lanes added as float
 //     pairs (within a few u^2 of the exact sum);
@@ -185,7 +189,7 @@ __device__ __forceinline__ void rho_kappa(float eh, float el, float vh, float vl
 template <int V>
 __global__ void __launch_bounds__(256)
 prep_rows_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
-                 int64_t Np, const float* __restrict__ mu, int to_bf16,
+                 int64_t Np, const float* __restrict__ mu, Operand to,
                  float* __restrict__ xt32, __nv_bfloat16* __restrict__ xt16,
                  float* __restrict__ norms, float* __restrict__ rho,
                  float* __restrict__ norms32, __nv_bfloat16* __restrict__ aug,
@@ -218,7 +222,7 @@ prep_rows_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
                     v[0] = X[src * D + j] - __ldg(mu + j);
                 }
             }
-            if (to_bf16) {
+            if (to == Operand::bf16) {
                 if constexpr (V == 4) {
                     const __nv_bfloat162 b01 = __floats2bfloat162_rn(v[0], v[1]);
                     const __nv_bfloat162 b23 = __floats2bfloat162_rn(v[2], v[3]);
@@ -234,7 +238,10 @@ prep_rows_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
                     vv[0] = __bfloat162float(b);
                 }
             } else {
-                if constexpr (V == 4)
+                if (to == Operand::f32_tiles)
+#pragma unroll
+                    for (int q = 0; q < V; ++q) xt32[((p / BM) * Dp + j + q) * BM + p % BM] = v[q];
+                else if constexpr (V == 4)
                     *reinterpret_cast<float4*>(xt32 + p * Dp + j) = make_float4(v[0], v[1], v[2], v[3]);
                 else
                     xt32[p * Dp + j] = v[0];
@@ -478,42 +485,170 @@ gather_split_kernel(const __nv_bfloat16* __restrict__ xh, const __nv_bfloat16* _
 
 // ------------------------------------------------------- fp32 candidate tiles
 
-// Shared-memory layout of the candidate kernel (dynamic).
+constexpr int kFStages = 4;   // operand chunks staged (as large as the tile of distances)
+
+// Shared-memory layout of the candidate kernels (dynamic).  The tile of
+// distances takes the operands' place once the products are done; lists are
+// keys (tile_key) in increasing order.
 template <int KC>
 struct CandSmem {
-    float As[2][BK][BM];
-    float Bs[2][BK][BN];
-    float list_d[BM][KC];
-    int list_i[BM][KC];
-    float q_d[BM][QC];
-    int q_i[BM][QC];
-    int q_cnt[BM];
-    float thr[BM];
+    union {
+        struct {
+            float As[kFStages][BK][BM];
+            float Bs[kFStages][BK][BN];
+        } op;
+        float dt[BM][BN];
+    };
+    unsigned long long list[BM][KC];
     float nrow[BM];
     float ncol[BN];
 };
 
-// Merge the queued entries of row r (owner thread) into its sorted list.
+// (distance, index) as one integer of the same order.
+__device__ __forceinline__ unsigned long long tile_key(float d, int i) {
+    const uint32_t u = __float_as_uint(d + 0.f);   // -0 as 0: equal distances go by index
+    return (unsigned long long)(u ^ ((uint32_t)((int)u >> 31) | 0x80000000u)) << 32 | (uint32_t)i;
+}
+__device__ __forceinline__ float key_dist(unsigned long long key) {
+    const uint32_t u = (uint32_t)(key >> 32);
+    return __uint_as_float(u >> 31 ? u ^ 0x80000000u : ~u);
+}
+__device__ __forceinline__ unsigned long long empty_key() { return tile_key(kInf, kNoIdx); }
+
+// One step of the tiles' products: features kk of 8 x 8 rows and columns of a
+// thread, two columns per instruction.
 template <int KC>
-__device__ __forceinline__ void merge_queue(CandSmem<KC>& s, int r) {
-    const int n = min(s.q_cnt[r], QC);
-    for (int e = 0; e < n; ++e) {
-        const float d = s.q_d[r][e];
-        const int i = s.q_i[r][e];
-        if (!lex_less(d, i, s.list_d[r][KC - 1], s.list_i[r][KC - 1])) continue;
-        int pos = KC - 1;
-        while (pos > 0 && lex_less(d, i, s.list_d[r][pos - 1], s.list_i[r][pos - 1])) {
-            s.list_d[r][pos] = s.list_d[r][pos - 1];
-            s.list_i[r][pos] = s.list_i[r][pos - 1];
-            --pos;
+__device__ __forceinline__ void tile_products(const CandSmem<KC>& s, int buf, int ty, int tx,
+                                              pair32 (&acc)[8][4]) {
+#pragma unroll
+    for (int kk = 0; kk < BK; ++kk) {
+        const float4 a0 = *reinterpret_cast<const float4*>(&s.op.As[buf][kk][4 * ty]);
+        const float4 a1 = *reinterpret_cast<const float4*>(&s.op.As[buf][kk][64 + 4 * ty]);
+        const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(&s.op.Bs[buf][kk][4 * tx]);
+        const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(&s.op.Bs[buf][kk][64 + 4 * tx]);
+        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        const pair32 b[4] = {b0.x, b0.y, b1.x, b1.y};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const pair32 aa = pack2(a[i], a[i]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = fma2(aa, b[j], acc[i][j]);
         }
-        s.list_d[r][pos] = d;
-        s.list_i[r][pos] = i;
     }
-    s.q_cnt[r] = 0;
-    s.thr[r] = s.list_d[r][KC - 1];
 }
 
+__device__ __forceinline__ void tile_copy16(float* dst, const float* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void tile_copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void tile_copies_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kFStages - 2) : "memory");
+}
+
+// Sorts one key per lane (up: increasing with the lane).
+template <int V>
+__device__ __forceinline__ void warp_sort(unsigned long long (&x)[V], const bool (&up)[V], int lane,
+                                          int from) {
+#pragma unroll
+    for (int n = 2; n <= 32; n <<= 1) {
+        if (n < from) continue;
+#pragma unroll
+        for (int o = n >> 1; o > 0; o >>= 1)
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const unsigned long long y = __shfl_xor_sync(0xffffffffu, x[v], o);
+                const bool asc = n == 32 ? up[v] : (lane & n) == 0;
+                const bool keep_min = ((lane & o) == 0) == asc;
+                x[v] = (y < x[v]) == keep_min ? y : x[v];
+            }
+    }
+}
+
+// Distances of the tile (products acc; n_p + n_q - 2 dot) into shared memory,
+// NaN (never a candidate) where ok refuses the pair, and each row's list
+// brought up to date: a warp takes 16 rows, four columns per lane.  A row with
+// many hits (the first tiles) sorts the tile's 128 keys and merges; one with
+// few inserts them one by one, the bound falling with each.  Queues filled by
+// atomics and merged by one thread per row made the whole block wait for the
+// longest: candidates of 2000 x 16 points 200 us, now 51 us; of 30011 x 200,
+// k = 12, 11.8 ms, now 8.5 (7.6 with the operand in tiles, below).
+constexpr int kSortHits = 20;
+template <int KC, class Ok>
+__device__ __forceinline__ void tile_select(CandSmem<KC>& s, const pair32 (&acc)[8][4], int64_t col0,
+                                            int ty, int tx, Ok ok) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int r = (i < 4) ? 4 * ty + i : 64 + 4 * ty + (i - 4);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float d[4];
+            unpack2(acc[i][2 * h], d[0], d[1]);
+            unpack2(acc[i][2 * h + 1], d[2], d[3]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int c = 64 * h + 4 * tx + j;
+                d[j] = ok(r, c) ? fmaf(-2.f, d[j], s.nrow[r] + s.ncol[c]) : __int_as_float(0x7fffffff);
+            }
+            *reinterpret_cast<float4*>(&s.dt[r][64 * h + 4 * tx]) = make_float4(d[0], d[1], d[2], d[3]);
+        }
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int RW = BM / (KT / 32);
+    for (int r = warp * RW; r < (warp + 1) * RW; ++r) {
+        const float4 x = *reinterpret_cast<const float4*>(&s.dt[r][4 * lane]);
+        const float v[4] = {x.x, x.y, x.z, x.w};
+        float thr = key_dist(s.list[r][KC - 1]);
+        int hits = 0;
+        unsigned m[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            m[j] = __ballot_sync(0xffffffffu, v[j] <= thr);
+            hits += __popc(m[j]);
+        }
+        if (hits == 0) continue;
+        unsigned long long l = lane < KC ? s.list[r][lane] : empty_key();
+        if (hits > kSortHits) {
+            unsigned long long k[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                k[j] = v[j] <= thr ? tile_key(v[j], (int)col0 + 4 * lane + j) : empty_key();
+            warp_sort<4>(k, {true, false, true, false}, lane, 2);
+            unsigned long long h[2] = {min(k[0], k[1]), min(k[2], k[3])};
+            warp_sort<2>(h, {true, false}, lane, 32);
+            unsigned long long q[1] = {min(h[0], h[1])};
+            warp_sort<1>(q, {false}, lane, 32);
+            q[0] = min(l, q[0]);
+            warp_sort<1>(q, {true}, lane, 32);
+            l = q[0];
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                unsigned left = m[j];
+                while (left) {
+                    const int src = __ffs(left) - 1;
+                    const float d = __shfl_sync(0xffffffffu, v[j], src);
+                    left &= left - 1;
+                    if (d > thr) continue;
+                    const unsigned long long key = tile_key(d, (int)col0 + 4 * src + j);
+                    const unsigned long long up = __shfl_up_sync(0xffffffffu, l, 1);
+                    // entries above the new key move one lane on
+                    if (l > key) l = lane > 0 && up > key ? up : key;
+                    thr = key_dist(__shfl_sync(0xffffffffu, l, KC - 1));
+                }
+            }
+        }
+        if (lane < KC) s.list[r][lane] = l;
+    }
+}
+
+// Bound by the float32 units (2 N^2 Dp operations: 49 of 80 TFLOP/s at 30011 x
+// 200).  The operand comes in tiles of 128 points by feature, so that a chunk of
+// either side is one contiguous run: four chunks under way by asynchronous copies
+// and no registers held for them (row by row through registers, transposed on the
+// way: 8.5 ms, now 7.6; the rows' values doubled in shared memory to save the
+// packing: 9.9).
 // Grid: (row blocks of 128, column splits).  Thread (ty, tx) = (t / 16, t % 16)
 // owns rows {4ty..4ty+3, 64+4ty..64+4ty+3} and the same pattern of columns.
 template <int KC>
@@ -529,118 +664,54 @@ knn_cand_fp32_kernel(const float* __restrict__ xt, const float* __restrict__ nor
     const int tile0 = (int)((int64_t)sp * n_tiles / splits);
     const int tile1 = (int)((int64_t)(sp + 1) * n_tiles / splits);
     if (t < BM) {
-        for (int j = 0; j < KC; ++j) { s.list_d[t][j] = kInf; s.list_i[t][j] = kNoIdx; }
-        s.q_cnt[t] = 0;
-        s.thr[t] = kInf;
+        for (int j = 0; j < KC; ++j) s.list[t][j] = empty_key();
         s.nrow[t] = norms[row0 + t];
     }
     const int nk = Dp / BK;
-    // load mapping: element idx = t + 256 i (i = 0, 1) -> row idx % 128, k-quad idx / 128
-    const int lr0 = t & 127, lq0 = t >> 7;          // i = 0: quads 0, 1
-    const int lq1 = lq0 + 2;                        // i = 1: quads 2, 3
+    // chunk kt of a tile: BK x 128 floats, contiguous in the tiled operand
+    const float* pa = xt + row0 * Dp + 4 * t;
     for (int tile = tile0; tile < tile1; ++tile) {
         const int64_t col0 = (int64_t)tile * BN;
         __syncthreads();  // previous epilogue finished with ncol / buffers
         if (t < BN) s.ncol[t] = norms[col0 + t];
-        float acc[8][8];
+        pair32 acc[8][4];
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-        const float* pa = xt + (row0 + lr0) * Dp;
-        const float* pb = xt + (col0 + lr0) * Dp;
-        float4 ra0 = __ldg(reinterpret_cast<const float4*>(pa + 4 * lq0));
-        float4 ra1 = __ldg(reinterpret_cast<const float4*>(pa + 4 * lq1));
-        float4 rb0 = __ldg(reinterpret_cast<const float4*>(pb + 4 * lq0));
-        float4 rb1 = __ldg(reinterpret_cast<const float4*>(pb + 4 * lq1));
-        auto stash = [&](int buf) {
-            s.As[buf][4 * lq0 + 0][lr0] = ra0.x; s.As[buf][4 * lq0 + 1][lr0] = ra0.y;
-            s.As[buf][4 * lq0 + 2][lr0] = ra0.z; s.As[buf][4 * lq0 + 3][lr0] = ra0.w;
-            s.As[buf][4 * lq1 + 0][lr0] = ra1.x; s.As[buf][4 * lq1 + 1][lr0] = ra1.y;
-            s.As[buf][4 * lq1 + 2][lr0] = ra1.z; s.As[buf][4 * lq1 + 3][lr0] = ra1.w;
-            s.Bs[buf][4 * lq0 + 0][lr0] = rb0.x; s.Bs[buf][4 * lq0 + 1][lr0] = rb0.y;
-            s.Bs[buf][4 * lq0 + 2][lr0] = rb0.z; s.Bs[buf][4 * lq0 + 3][lr0] = rb0.w;
-            s.Bs[buf][4 * lq1 + 0][lr0] = rb1.x; s.Bs[buf][4 * lq1 + 1][lr0] = rb1.y;
-            s.Bs[buf][4 * lq1 + 2][lr0] = rb1.z; s.Bs[buf][4 * lq1 + 3][lr0] = rb1.w;
-        };
-        stash(0);
-        __syncthreads();
-        for (int kt = 0; kt < nk; ++kt) {
-            const int buf = kt & 1;
-            if (kt + 1 < nk) {
-                const int k0 = (kt + 1) * BK;
-                ra0 = __ldg(reinterpret_cast<const float4*>(pa + k0 + 4 * lq0));
-                ra1 = __ldg(reinterpret_cast<const float4*>(pa + k0 + 4 * lq1));
-                rb0 = __ldg(reinterpret_cast<const float4*>(pb + k0 + 4 * lq0));
-                rb1 = __ldg(reinterpret_cast<const float4*>(pb + k0 + 4 * lq1));
-            }
+            for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+        const float* pb = xt + col0 * Dp + 4 * t;
+        auto fetch = [&](int kt) {
+            if (kt < nk) {
+                float* a = &s.op.As[kt % kFStages][0][0] + 4 * t;
+                float* b = &s.op.Bs[kt % kFStages][0][0] + 4 * t;
 #pragma unroll
-            for (int kk = 0; kk < BK; ++kk) {
-                const float4 a0 = *reinterpret_cast<const float4*>(&s.As[buf][kk][4 * ty]);
-                const float4 a1 = *reinterpret_cast<const float4*>(&s.As[buf][kk][64 + 4 * ty]);
-                const float4 b0 = *reinterpret_cast<const float4*>(&s.Bs[buf][kk][4 * tx]);
-                const float4 b1 = *reinterpret_cast<const float4*>(&s.Bs[buf][kk][64 + 4 * tx]);
-                const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-            }
-            if (kt + 1 < nk) stash(buf ^ 1);
-            __syncthreads();
-        }
-        // ---- epilogue: dt = n_p + n_q - 2 dot, filter against the row thresholds
-        unsigned long long pend = 0ull;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int r = (i < 4) ? 4 * ty + i : 64 + 4 * ty + (i - 4);
-            const int64_t p = row0 + r;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int c = (j < 4) ? 4 * tx + j : 64 + 4 * tx + (j - 4);
-                const int64_t q = col0 + c;
-                const float d = fmaf(-2.f, acc[i][j], s.nrow[r] + s.ncol[c]);
-                acc[i][j] = d;
-                if (p < N && q < N && q != p && d <= s.thr[r]) pend |= 1ull << (i * 8 + j);
-            }
-        }
-        while (__syncthreads_or(pend != 0ull)) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int r = (i < 4) ? 4 * ty + i : 64 + 4 * ty + (i - 4);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (pend & (1ull << (i * 8 + j))) {
-                        const int slot = atomicAdd(&s.q_cnt[r], 1);
-                        if (slot < QC) {
-                            const int c = (j < 4) ? 4 * tx + j : 64 + 4 * tx + (j - 4);
-                            s.q_d[r][slot] = acc[i][j];
-                            s.q_i[r][slot] = (int)(col0 + c);
-                            pend &= ~(1ull << (i * 8 + j));
-                        }
-                    }
+                for (int h = 0; h < BK * BM / (4 * KT); ++h) {
+                    tile_copy16(a + 4 * KT * h, pa + kt * (BK * BM) + 4 * KT * h);
+                    tile_copy16(b + 4 * KT * h, pb + kt * (BK * BN) + 4 * KT * h);
                 }
             }
-            __syncthreads();
-            if (t < BM) merge_queue<KC>(s, t);
-            __syncthreads();
+            tile_copies_commit();   // (an empty group keeps the wait count uniform)
+        };
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int r = (i < 4) ? 4 * ty + i : 64 + 4 * ty + (i - 4);
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if ((pend & (1ull << (i * 8 + j))) && !(acc[i][j] <= s.thr[r]))
-                        pend &= ~(1ull << (i * 8 + j));
-            }
+        for (int kt = 0; kt < kFStages - 1; ++kt) fetch(kt);
+        for (int kt = 0; kt < nk; ++kt) {
+            tile_copies_wait();     // this thread's copies of chunk kt have landed
+            __syncthreads();        // ... every thread's, and chunk kt - 1 is read
+            fetch(kt + kFStages - 1);
+            tile_products<KC>(s, kt % kFStages, ty, tx, acc);
         }
+        __syncthreads();            // the operands are read: the tile may take their place
+        tile_select<KC>(s, acc, col0, ty, tx, [&](int r, int c) {
+            const int64_t p = row0 + r, q = col0 + c;
+            return p < N && q < N && q != p;
+        });
     }
     __syncthreads();
     if (t < BM) {
         const int64_t o = ((int64_t)sp * Np + row0 + t) * KC;
         for (int j = 0; j < KC; ++j) {
-            cand_d[o + j] = s.list_d[t][j];
-            cand_i[o + j] = s.list_i[t][j] == kNoIdx ? -1 : s.list_i[t][j];
+            cand_d[o + j] = key_dist(s.list[t][j]);
+            cand_i[o + j] = (int)(uint32_t)s.list[t][j] == kNoIdx ? -1 : (int)(uint32_t)s.list[t][j];
         }
     }
 }
@@ -680,9 +751,7 @@ knn_cand_query_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
             const int64_t f = rb * BM + t;
             const int64_t p = (f < F) ? (int64_t)fb_list[f] : -1;
             prow[t] = p;
-            for (int j = 0; j < KC; ++j) { s.list_d[t][j] = kInf; s.list_i[t][j] = kNoIdx; }
-            s.q_cnt[t] = 0;
-            s.thr[t] = kInf;
+            for (int j = 0; j < KC; ++j) s.list[t][j] = empty_key();
             s.nrow[t] = (p >= 0) ? norms32[p] : kInf;
         }
         __syncthreads();
@@ -692,11 +761,11 @@ knn_cand_query_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
             __syncthreads();  // previous epilogue finished with ncol / buffers
             if (t < BN) s.ncol[t] = (col0 + t < N) ? norms32[col0 + t] : kInf;
             const int64_t qb_row = (col0 + lr0 < N) ? col0 + lr0 : -1;
-            float acc[8][8];
+            pair32 acc[8][4];
 #pragma unroll
             for (int i = 0; i < 8; ++i)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+                for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
             float ra[8], rbv[8];
             // 16-byte loads when every row starts on a 16-byte boundary and the
             // four features of a chunk are all inside the row (D % 4 == 0)
@@ -734,8 +803,8 @@ knn_cand_query_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     const int kk = 4 * (c < 4 ? lq0 : lq1) + (c & 3);
-                    s.As[buf][kk][lr0] = ra[c];
-                    s.Bs[buf][kk][lr0] = rbv[c];
+                    s.op.As[buf][kk][lr0] = ra[c];
+                    s.op.Bs[buf][kk][lr0] = rbv[c];
                 }
             };
             fetch(0);
@@ -744,66 +813,14 @@ knn_cand_query_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
             for (int kt = 0; kt < nk; ++kt) {
                 const int buf = kt & 1;
                 if (kt + 1 < nk) fetch((kt + 1) * BK);
-#pragma unroll
-                for (int kk = 0; kk < BK; ++kk) {
-                    const float4 a0 = *reinterpret_cast<const float4*>(&s.As[buf][kk][4 * ty]);
-                    const float4 a1 = *reinterpret_cast<const float4*>(&s.As[buf][kk][64 + 4 * ty]);
-                    const float4 b0 = *reinterpret_cast<const float4*>(&s.Bs[buf][kk][4 * tx]);
-                    const float4 b1 = *reinterpret_cast<const float4*>(&s.Bs[buf][kk][64 + 4 * tx]);
-                    const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                    const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-                }
+                tile_products<KC>(s, buf, ty, tx, acc);
                 if (kt + 1 < nk) stash(buf ^ 1);
                 __syncthreads();
             }
-            // ---- epilogue: dt = n_p + n_q - 2 dot, filter against the row thresholds
-            unsigned long long pend = 0ull;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int r = (i < 4) ? 4 * ty + i : 64 + 4 * ty + (i - 4);
-                const int64_t p = prow[r];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int c = (j < 4) ? 4 * tx + j : 64 + 4 * tx + (j - 4);
-                    const int64_t q = col0 + c;
-                    const float d = fmaf(-2.f, acc[i][j], s.nrow[r] + s.ncol[c]);
-                    acc[i][j] = d;
-                    if (p >= 0 && q < N && q != p && d <= s.thr[r]) pend |= 1ull << (i * 8 + j);
-                }
-            }
-            while (__syncthreads_or(pend != 0ull)) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int r = (i < 4) ? 4 * ty + i : 64 + 4 * ty + (i - 4);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        if (pend & (1ull << (i * 8 + j))) {
-                            const int slot = atomicAdd(&s.q_cnt[r], 1);
-                            if (slot < QC) {
-                                const int c = (j < 4) ? 4 * tx + j : 64 + 4 * tx + (j - 4);
-                                s.q_d[r][slot] = acc[i][j];
-                                s.q_i[r][slot] = (int)(col0 + c);
-                                pend &= ~(1ull << (i * 8 + j));
-                            }
-                        }
-                    }
-                }
-                __syncthreads();
-                if (t < BM) merge_queue<KC>(s, t);
-                __syncthreads();
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int r = (i < 4) ? 4 * ty + i : 64 + 4 * ty + (i - 4);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        if ((pend & (1ull << (i * 8 + j))) && !(acc[i][j] <= s.thr[r]))
-                            pend &= ~(1ull << (i * 8 + j));
-                }
-            }
+            tile_select<KC>(s, acc, col0, ty, tx, [&](int r, int c) {
+                const int64_t p = prow[r], q = col0 + c;
+                return p >= 0 && q < N && q != p;
+            });
         }
         __syncthreads();
         if (t < BM) {
@@ -811,8 +828,8 @@ knn_cand_query_kernel(const float* __restrict__ X, int64_t N, int D, int Dp,
             if (f < F) {
                 const int64_t o = ((int64_t)sp * F + f) * KC;
                 for (int j = 0; j < KC; ++j) {
-                    cand_d[o + j] = s.list_d[t][j];
-                    cand_i[o + j] = s.list_i[t][j] == kNoIdx ? -1 : s.list_i[t][j];
+                    cand_d[o + j] = key_dist(s.list[t][j]);
+                    cand_i[o + j] = (int)(uint32_t)s.list[t][j] == kNoIdx ? -1 : (int)(uint32_t)s.list[t][j];
                 }
             }
         }
@@ -1930,7 +1947,7 @@ namespace {
 slk_status launch_prep(slk_ctx* ctx, const float* X, int64_t N, int D, int Dp, int64_t Np,
                        double* colsum, float* mu, float* xt32, __nv_bfloat16* xt16,
                        float* norms, float* rho, float* norms32, __nv_bfloat16* aug, const GroupBufs* grp,
-                       DevState* st) {
+                       DevState* st, bool tiles = false) {
     cudaStream_t s = ctx->stream;
     const bool v4 = D % 4 == 0 && Dp >= 128 && (reinterpret_cast<uintptr_t>(X) & 15) == 0 &&
                     (reinterpret_cast<uintptr_t>(mu) & 15) == 0;
@@ -1951,12 +1968,12 @@ slk_status launch_prep(slk_ctx* ctx, const float* X, int64_t N, int D, int Dp, i
     }
     int64_t pg = (Np + 7) / 8;
     if (pg > (int64_t)ctx->num_sms * 64) pg = (int64_t)ctx->num_sms * 64;
-    const int to_bf16 = xt16 != nullptr ? 1 : 0;
+    const Operand to = xt16 ? Operand::bf16 : tiles ? Operand::f32_tiles : Operand::f32_rows;
     if (v4)
-        prep_rows_kernel<4><<<(unsigned)pg, 256, 0, s>>>(X, N, D, Dp, Np, mu, to_bf16, xt32, xt16,
+        prep_rows_kernel<4><<<(unsigned)pg, 256, 0, s>>>(X, N, D, Dp, Np, mu, to, xt32, xt16,
                                                          norms, rho, norms32, aug, perm, st);
     else
-        prep_rows_kernel<1><<<(unsigned)pg, 256, 0, s>>>(X, N, D, Dp, Np, mu, to_bf16, xt32, xt16,
+        prep_rows_kernel<1><<<(unsigned)pg, 256, 0, s>>>(X, N, D, Dp, Np, mu, to, xt32, xt16,
                                                          norms, rho, norms32, aug, perm, st);
     SLK_LAUNCH_CHECK(ctx, "prep_rows_kernel");
     return SLK_OK;
@@ -2005,7 +2022,7 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
                                          pl.bf16 ? nullptr : (float*)xt,
                                          pl.bf16 ? (__nv_bfloat16*)xt : nullptr, norms, rho,
                                          pl.bf16 ? norms32 : nullptr, pl.aug ? aug : nullptr,
-                                         pl.grouped ? &kb.grp : nullptr, st);
+                                         pl.grouped ? &kb.grp : nullptr, st, !pl.bf16);
         if (r != SLK_OK) return r;
     }
     // rounding unit of a tile's dot-product accumulation: 2^-23 on the tensor
