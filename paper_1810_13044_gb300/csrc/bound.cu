@@ -970,12 +970,16 @@ __device__ __forceinline__ float rows_update_cached(int lr0, int lstride, int nr
     return dmax;
 }
 
-#ifndef SLK_BOUND_CACHED_RPG2
-#define SLK_BOUND_CACHED_RPG2 2
-#endif
+// Rows per group and blocks per SM.  Two labels per lane: one row per group and
+// four blocks (64 registers) rather than two rows and two blocks -- as many
+// loads in flight, and one warp's softmax covers another's gather.  40 updates
+// of 150001 points, L = 37, k = 7: 2.82 ms, now 2.20; 200 of 70000, L = 10,
+// k = 5: 2.00, now 1.76.  One label per lane: four rows (144 registers) hide
+// more than warps do (2000 points, L = 5: 0.052 ms; 0.087 with four blocks).
 template <int LPL>
 struct CachedTiling {
-    static constexpr int rpg = (LPL == 1) ? 4 : (LPL == 2 ? SLK_BOUND_CACHED_RPG2 : (LPL == 4 ? 2 : 1));
+    static constexpr int rpg = (LPL == 1) ? 4 : (LPL == 4 ? 2 : 1);
+    static constexpr int blocks = (LPL == 2) ? 4 : 1;
 };
 
 // Persistent inner loop over a fixed-degree graph (kdeg edges per row) with
@@ -983,7 +987,7 @@ struct CachedTiling {
 // [b rpc, (b + 1) rpc).  Same updates, barrier and results as
 // bound_persistent_kernel.
 template <int G, int LPL>
-__global__ void __launch_bounds__(kThreads, SLK_BOUND_MINB)
+__global__ void __launch_bounds__(kThreads, CachedTiling<LPL>::blocks)
 bound_cached_kernel(const float* __restrict__ A, const int32_t* __restrict__ col_idx,
                     const float* __restrict__ w, int64_t N, int L, float lambda, float* Z0,
                     float* Z1, int max_iters, float tol, int kdeg, int rpc, DevState* st) {
