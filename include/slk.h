@@ -83,7 +83,9 @@ const char* slk_last_error(const slk_ctx* ctx);
  *                      1, HEAT writes exp(-dist2 / (2 sigma^2)).
  *   affinity SLK_AFFINITY_*; sigma (> 0) is used by HEAT only.
  *   precision SLK_KNN_FP32: float32 SIMT distance tiles; SLK_KNN_BF16_RERANK:
- *            bfloat16 tensor-core (tcgen05) distance tiles.  Both produce
+ *            bfloat16 tensor-core (tcgen05) distance tiles (above a work size
+ *            over points sorted by region, without the tiles that cannot hold
+ *            a neighbour).  Both produce
  *            candidates that are re-ranked with exact float32 distances and
  *            certified by a rounding-error bound.  With BF16_RERANK the rows
  *            that fail it get two-term bfloat16 tensor-core tiles (each
@@ -248,8 +250,8 @@ slk_status slk_solve_host(slk_ctx* ctx, const float* X, int64_t N, int32_t D, in
  * D(x_0)^2 + ... + D(x_p)^2 exceeds u[i-1] * sum_q D(x_q)^2, where D(x)^2 is
  * the squared Euclidean distance to the closest of seeds[0..i-1] (float64
  * sums); the last point if no running sum does, and point floor(u[i-1] N) if
- * every D(x)^2 is 0.  Two launches per seed: a float64 distance pass over X
- * and a one-block selection.
+ * every D(x)^2 is 0.  One launch per seed: float64 distances of the points that
+ * the last seed may be nearest to, and the selection.
  *   X [N x D]; first in [0, N); u [host, L - 1] uniforms in [0, 1) (NULL
  *   allowed when L = 1); seeds [L] device int32 out.  1 <= L <= N.
  * Synchronises the context stream. */
@@ -411,7 +413,8 @@ slk_status slk_server_destroy(slk_server* srv);
 slk_status slk_server_submit(slk_server* srv, const slk_instance* req, int64_t* ticket);
 slk_status slk_server_step(slk_server* srv, int32_t* n_running, int32_t* n_queued);
 slk_status slk_server_poll(slk_server* srv, int64_t ticket, int32_t* state, slk_stats* stats);
-/* Arena bytes a request needs while its graph is built (its peak) [host out]. */
+/* Arena bytes a request needs at least while its graph is built (its peak) [host
+ * out]; where the arena has more, the graph's scratch takes more. */
 slk_status slk_server_request_bytes(slk_server* srv, const slk_instance* req, int64_t* bytes);
 
 /* slk_bound_iterate for callers that cannot allocate device memory.  The

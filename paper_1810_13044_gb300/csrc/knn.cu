@@ -8,10 +8,13 @@
 //     perturbation rho_p >= ||xt_p - (x_p - mu)|| (float32 lane sums with
 //     their rounding bounds, lanes added as 2Sum float pairs).
 //  2. candidates: a distance-tile kernel evaluates
-//     dt(p, q) = ||xt_p||^2 + ||xt_q||^2 - 2 xt_p . xt_q for all pairs and keeps,
-//     per row and per column split, the KC smallest (KC > k), sorted.
-//  3. rerank + certificate (one warp per row): merge the splits' sorted lists,
-//     recompute exactly in float32, from the original features, the distances
+//     dt(p, q) = ||xt_p||^2 + ||xt_q||^2 - 2 xt_p . xt_q.  float32: for all pairs,
+//     keeping per row and per column split the KC smallest (KC > k), sorted.
+//     bfloat16 (knn_sweep.cu): keeping what a threshold from the k-th smallest
+//     lets through, unsorted; above a work size over points sorted by region
+//     (knn_group.cu) and only the tiles that can hold a neighbour.
+//  3. rerank + certificate (one warp per row; knn_rerank_kernel, for the sweep's
+//     slots knn_select_kernel): rank the candidates, recompute exactly in float32, from the original features, the distances
 //     of the candidates whose lower bound can still reach the k nearest, keep
 //     the k smallest.  With T the KC-th smallest dt, every other point q
 //     satisfies dt(p,q) >= T, hence (rounding bounds below) its true distance
@@ -19,8 +22,8 @@
 //     certified when the k-th exact distance, inflated by its own rounding
 //     bound, is below LB; then the row equals a full float32 scan.
 //  4. fallback: with bfloat16 candidates, the rows that fail the certificate
-//     first get float32 candidate tiles and the same rerank under the float32
-//     certificate; rows that fail that (or the float32 certificate of a
+//     get two-term bfloat16 tiles from 100000 points on, then float32 candidate
+//     tiles, each under its own certificate; rows that fail that (or the float32 certificate of a
 //     float32 pass) are rescanned exactly.
 #include <cuda_bf16.h>
 #include <math.h>
