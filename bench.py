@@ -488,7 +488,8 @@ def measure_workload(W, args, ctx, dev, world, stream, main: bool):
         "initial_modes": None if init_ms is None else {
             "ms": init_ms, "bound": "alu",
             "achieved_tflops": 2.0 * N * N * D / (init_ms / 1e3) / 1e12, "peak_tflops": fp32_peak,
-            "algorithmic": "2*N*N*D flop (float32 distance tiles) + N*N exp"},
+            "algorithmic": "2*N*N*D flop (float32 distance tiles) + N*N exp; all pairs counted, the "
+                           "tiles that cannot hold a cluster's maximiser are left out"},
         "phase_ms_per_step": {k_: v / args.steps for k_, v in ms_phase.items()},
         "roofline": roof,
         "roofline_bound": roof_bound,
