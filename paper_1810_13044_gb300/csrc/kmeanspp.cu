@@ -152,7 +152,7 @@ __device__ void kpp_select(const KppArgs& a, int i) {
         for (int w = 0; w < (t >> 5); ++w) excl += wt[w];
     }
     if (t == kTile - 1) s_total = incl;
-    if (t == 0) s_pos = kTile;
+    if (t == 0) { s_pos = kTile; s_last = 0; }
     __syncthreads();
     const double total = s_total, r_u = a.u[i - 1], r = r_u * total;
     if (!(total > 0.0)) {
@@ -160,9 +160,15 @@ __device__ void kpp_select(const KppArgs& a, int i) {
         if (t == 0) a.seeds[i] = (int32_t)(pick < a.N - 1 ? pick : a.N - 1);
         return;
     }
-    if (incl > r) atomicMin(&s_pos, t);
+    // only strips that hold something: each lane of the scan adds in an order of
+    // its own, so a prefix may round up across empty strips (those past n_tiles
+    // among them), or the last one that counts may round below r
+    if (strip > 0.0) {
+        if (incl > r) atomicMin(&s_pos, t);
+        atomicMax(&s_last, t);
+    }
     __syncthreads();
-    const int owner = s_pos;
+    const int owner = s_pos < kTile ? s_pos : r < total ? s_last : kTile;
     if (owner >= kTile) {   // no running sum exceeds r
         if (t == 0) a.seeds[i] = (int32_t)(a.N - 1);
         return;
@@ -175,8 +181,11 @@ __device__ void kpp_select(const KppArgs& a, int i) {
         int tile = -1, last = b;
         for (int j = b; j < e && tile < 0; ++j) {
             const double s = __ldcg(a.tile_sum + j);
-            if (s > 0.0) { last = j; off = run; }
-            if (run + s > r) tile = j;
+            if (s > 0.0) {
+                last = j;
+                off = run;
+                if (run + s > r) tile = j;
+            }
             run += s;
         }
         s_off = off;

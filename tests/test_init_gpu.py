@@ -217,3 +217,19 @@ def test_initial_modes_other_clusters_left_out(slk, N, D, L, sigma):
     g_modes, g_assign, g_dens = slk.initial_modes(dev(X), dev(seeds), sigma)
     _check_assign(X, seeds, host(g_assign), o_assign)
     _check_modes(X, sigma, host(g_modes), np.array(g_dens), o_modes, o_dens, o_assign)
+
+
+@pytest.mark.parametrize("N,tail", [(2100, 0), (2304, 0), (2304, 700), (5000, 0), (5000, 1500), (3000, 100),
+                                    (70001, 300)])
+def test_kmeanspp_largest_draw(slk, N, tail):
+    """A draw just below 1 asks for the last point away from seed 0, whichever
+    way the prefix sums round: never a point past the end, nor one of the `tail`
+    last points, which coincide with it."""
+    u = [1.0 - 2.0 ** -53]
+    for seed in range(40):
+        X = inputs.rng(seed).normal(size=(N, 1)).astype(np.float32)
+        if tail:
+            X[-tail:] = X[0]
+        want = oracle.kmeanspp(X, 2, 0, u)
+        assert want[1] == np.nonzero(X[:, 0] != X[0, 0])[0][-1]
+        np.testing.assert_array_equal(host(slk.kmeanspp(dev(X), 2, 0, u)), want)
