@@ -268,7 +268,8 @@ kpp_step_kernel(const KppArgs a, int i) {
                 const double d = exact64<VEC4, G>(a.X + (p0 + at) * a.D, c, a.D, sub);
                 if (sub == 0 && k < ne) {
                     const int64_t q = p0 + at;
-                    if (i == 1 || d < a.closest[q]) {
+                    // (a distance takes the place of a NaN, inf - inf to an earlier seed)
+                    if (i == 1 || d < a.closest[q] || isnan(a.closest[q])) {
                         a.closest[q] = d;
                         a.closest_up[q] = __double2float_ru(d);
                         a.own[q] = i - 1;

@@ -233,3 +233,15 @@ def test_kmeanspp_largest_draw(slk, N, tail):
         want = oracle.kmeanspp(X, 2, 0, u)
         assert want[1] == np.nonzero(X[:, 0] != X[0, 0])[0][-1]
         np.testing.assert_array_equal(host(slk.kmeanspp(dev(X), 2, 0, u)), want)
+
+
+@pytest.mark.parametrize("D", [3, 40])
+def test_kmeanspp_infinite_first_seed(slk, D):
+    """Seed 0 with an infinite feature: its distance to itself is not a number,
+    so the first draw goes by place; its distance to seed 1 is infinite, so from
+    then on no running sum exceeds u times the total and the last point is taken."""
+    N = 1001
+    X = inputs.rng(D).normal(size=(N, D)).astype(np.float32)
+    X[5, 1] = np.inf
+    got = host(slk.kmeanspp(dev(X), 4, 5, [0.25, 0.5, 0.75]))
+    np.testing.assert_array_equal(got, [5, 250, N - 1, N - 1])
