@@ -360,12 +360,16 @@ density_depth_kernel(const float* __restrict__ d2, const int32_t* __restrict__ p
     __syncthreads();
     for (int l = 0; l < L; ++l) {
         const float dl = d2[y * L + l], ds = d2[(int64_t)seeds[l] * L + j];
-        float h = -__int_as_float(0x7f800000);   // no border: nothing is known
-        if (l != j && ds > 1e-20f) h = (dl - dj - 4e-6f * (dl + dj)) / (2.00001f * sqrtf(ds));
+        // without a border, and where a squared distance overflows float32 (inf -
+        // inf, finite / inf), nothing is known
+        const float inf = __int_as_float(0x7f800000);
+        float h = -inf;
+        if (l != j && ds > 1e-20f && ds < inf) h = (dl - dj - 4e-6f * (dl + dj)) / (2.00001f * sqrtf(ds));
+        if (!(h == h)) h = -inf;
         if (h < 0.f) h *= 1.0001f;
         if (in) {
-            const float k = fminf(floorf(h * inv), (float)(kDepthBins - 33));   // at most the last place
-            atomicAdd(&bins[k > -32.f ? (int)k + 32 : 0], 1);
+            const float k = floorf(h * inv);
+            atomicAdd(&bins[k > -32.f ? (int)fminf(k, (float)(kDepthBins - 33)) + 32 : 0], 1);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) h = fminf(h, __shfl_xor_sync(0xffffffffu, h, o));

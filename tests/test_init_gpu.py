@@ -235,6 +235,35 @@ def test_kmeanspp_largest_draw(slk, N, tail):
         np.testing.assert_array_equal(host(slk.kmeanspp(dev(X), 2, 0, u)), want)
 
 
+def test_initial_modes_distances_beyond_float32(slk):
+    """Squared distances to both seeds that overflow float32 say nothing about
+    the side of the border a point lies on.  Cluster 0 is its seed and a shell
+    whose distances overflow; the shell's densest place is a point of cluster 1
+    near its centre (every distance of that one, and their sums, are finite)."""
+    U, D, n = 1e19, 64, 300
+    sig = float(np.sqrt(0.72)) * U
+    g = inputs.rng(17)
+    shell = np.zeros((n, D))
+    shell[:, 2:] = g.normal(size=(n, D - 2))
+    shell *= 1.2 / np.linalg.norm(shell, axis=1, keepdims=True)
+    shell[:, 1] = -0.05
+    s0, s1, y = np.zeros((3, D))
+    s0[:2], s1[:2], y[:2] = (1.45, -0.3), (1.45, 0.3), (0.2, 0.05)
+    near1 = s1 + 0.001 * g.normal(size=(20, D))
+    X = (U * np.concatenate([s0[None], s1[None], y[None], near1, shell])).astype(np.float32)
+    seeds = np.array([0, 1], np.int32)
+    X64 = X.astype(np.float64)
+    d2 = np.stack([((X64 - X64[s]) ** 2).sum(1) for s in seeds], 1)
+    top = float(np.finfo(np.float32).max)
+    assert (d2[-n:] > top).all() and (d2[:-n].sum(1) < top).all()
+    o_modes, o_assign, o_dens = oracle.initial_modes(X, seeds, sig)
+    assert o_modes[0] == 2 and o_assign[2] == 1 and (o_assign[-n:] == 0).all()
+    g_modes, g_assign, g_dens = slk.initial_modes(dev(X), dev(seeds), sig)
+    np.testing.assert_array_equal(host(g_assign), o_assign)
+    assert host(g_modes)[0] == 2
+    _check_modes(X, sig, host(g_modes), np.array(g_dens), o_modes, o_dens, o_assign)
+
+
 @pytest.mark.parametrize("D", [3, 40])
 def test_kmeanspp_infinite_first_seed(slk, D):
     """Seed 0 with an infinite feature: its distance to itself is not a number,
