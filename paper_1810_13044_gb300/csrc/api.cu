@@ -27,6 +27,9 @@ slk_status cuda_err(slk_ctx* ctx, cudaError_t e, const char* where) {
     return set_err(ctx, st, "%s: %s (%s)", where, cudaGetErrorName(e), cudaGetErrorString(e));
 }
 
+// Bytes allocated for a workspace of `bytes`.
+static size_t ws_rounded(size_t bytes) { return align_up(bytes + bytes / 8, 1 << 20); }
+
 slk_status ensure_ws(slk_ctx* ctx, size_t bytes) {
     if (bytes <= ctx->ws_bytes) return SLK_OK;
     if (ctx->ws) {
@@ -36,7 +39,7 @@ slk_status ensure_ws(slk_ctx* ctx, size_t bytes) {
         ctx->ws = nullptr;
         ctx->ws_bytes = 0;
     }
-    const size_t want = align_up(bytes + bytes / 8, 1 << 20);
+    const size_t want = ws_rounded(bytes);
     cudaError_t e = cudaMalloc(&ctx->ws, want);
     if (e != cudaSuccess) {
         ctx->ws = nullptr;
@@ -50,11 +53,23 @@ slk_status ensure_ws(slk_ctx* ctx, size_t bytes) {
 slk_status ensure_ws_of(slk_ctx* ctx, size_t want, size_t least, bool* full) {
     *full = true;
     if (want <= ctx->ws_bytes) return SLK_OK;
-    if (want < ctx->ws_refused) {
+    // a refused size is asked for again once more memory is free than at the
+    // refusal (the workspace itself counts as free: a larger one replaces it)
+    size_t avail = 0, total = 0;
+    bool ask = want < ctx->ws_refused;
+    if (!ask) {
+        SLK_CUDA_TRY(ctx, cudaMemGetInfo(&avail, &total));
+        avail += ctx->ws_bytes;
+        ask = avail >= ws_rounded(want) && avail > ctx->ws_refused_avail;
+    }
+    if (ask) {
         const slk_status r = ensure_ws(ctx, want);
+        if (r == SLK_OK) ctx->ws_refused = SIZE_MAX;
         if (r != SLK_ERR_OOM) return r;
-        ctx->ws_refused = want;
         ctx->err.clear();
+        SLK_CUDA_TRY(ctx, cudaMemGetInfo(&avail, &total));   // the old workspace is freed
+        ctx->ws_refused = want;
+        ctx->ws_refused_avail = avail;
     }
     *full = false;
     return ensure_ws(ctx, least);

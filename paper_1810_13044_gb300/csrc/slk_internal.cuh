@@ -21,7 +21,8 @@ struct slk_ctx {
     // scratch workspace, grown on demand (cudaMalloc), freed by slk_destroy
     void* ws = nullptr;
     size_t ws_bytes = 0;
-    size_t ws_refused = SIZE_MAX;   // smallest size that could not be allocated
+    size_t ws_refused = SIZE_MAX;   // last size that could not be allocated ...
+    size_t ws_refused_avail = 0;    // ... and the memory that was free then
     // small pinned host block for scalar results
     void* host_pin = nullptr;
     // small device block for scalar state (status words, sigma, energy)
@@ -104,8 +105,8 @@ slk_status set_err(slk_ctx* ctx, slk_status st, const char* fmt, ...);
 slk_status cuda_err(slk_ctx* ctx, cudaError_t e, const char* where);
 // Make sure ctx->ws holds at least `bytes`; returns SLK_OK or SLK_ERR_OOM.
 slk_status ensure_ws(slk_ctx* ctx, size_t bytes);
-// The same for `want` bytes, or for `least` where so much cannot be had (asked
-// for only once per size); *full: whether there are `want`.
+// The same for `want` bytes, or for `least` where so much cannot be had; *full:
+// whether there are `want`.
 slk_status ensure_ws_of(slk_ctx* ctx, size_t want, size_t least, bool* full);
 
 #define SLK_CUDA_TRY(ctx, expr)                                                  \

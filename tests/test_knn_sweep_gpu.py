@@ -98,3 +98,44 @@ def test_least_workspace_gives_the_same_solution(slk):
     assert s0["sigma"] == s1["sigma"]
     big.close()
     small.close()
+
+
+def test_refused_workspace_is_asked_for_again(slk):
+    """A context that once could not have the larger workspace takes the least
+    one, and the larger one once the memory is free again."""
+    N, D, k = 200000, 64, 10
+    MB = 1 << 20
+    X = torch.from_numpy(points("blobs", N, D, 1)).cuda()
+
+    def spare():                  # leaves room for the outputs in torch's cache
+        outs = [torch.empty(4 * N * k, device="cuda") for _ in range(2)]
+        del outs
+
+    def grown(ctx):               # device memory a graph takes beyond its outputs
+        free = torch.cuda.mem_get_info()[0]
+        g = slk.knn_graph(X, k, precision="bf16_rerank", ctx=ctx)
+        torch.cuda.synchronize()
+        return free - torch.cuda.mem_get_info()[0], g
+
+    a = slk.Context()
+    grown(a)                      # (first launches load code)
+    a.close()
+    a, b = slk.Context(), slk.Context()
+    spare()
+    full, g0 = grown(a)
+    a.close()
+    torch.cuda.empty_cache()
+    spare()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - (full - 24 * MB), dtype=torch.uint8, device="cuda")
+    try:
+        less, g1 = grown(b)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    assert 0 < less < full - 24 * MB
+    spare()
+    more, g2 = grown(b)
+    assert more > 24 * MB
+    for g in (g1, g2):
+        assert torch.equal(g.col_idx, g0.col_idx) and torch.equal(g.dist2, g0.dist2)
+    b.close()
