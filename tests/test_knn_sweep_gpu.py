@@ -100,6 +100,18 @@ def test_least_workspace_gives_the_same_solution(slk):
     small.close()
 
 
+def test_all_points_equal_sorted(slk):
+    """The same above the work size from which the points are sorted: no border
+    between any two pivots, and every row of the first sweep given up on ties."""
+    N, D, k = 40000, 40, 6
+    X = torch.from_numpy(points("equal", N, D, 0)).cuda()
+    g = slk.knn_graph(X, k, precision="bf16_rerank")
+    col = g.col_idx.cpu().numpy().reshape(N, k)
+    want = np.arange(k)[None, :] + (np.arange(k)[None, :] >= np.arange(N)[:, None])
+    np.testing.assert_array_equal(col, want)
+    assert float(g.dist2.abs().max()) == 0.0
+
+
 def test_refused_workspace_is_asked_for_again(slk):
     """A context that once could not have the larger workspace takes the least
     one, and the larger one once the memory is free again."""
