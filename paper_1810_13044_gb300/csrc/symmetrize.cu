@@ -7,16 +7,18 @@
 //   sym_in_count_kernel   in-degrees (atomic counts)
 //   scan (3 launches)     in-list offsets
 //   sym_in_fill_kernel    sources of every column (atomic cursors: any order)
-//   sym_sort_long_kernel  in-lists of more than kLongList entries, by the block
-//                         that finds them: every entry's rank by counting
-//   sym_rows_kernel<0>    per row: sort its in-list by source, sort a copy of
-//                         its out-list by column, count the union
+//   sym_rows_kernel<0>    per row: sort its in-list by source (more than
+//                         kLongList entries: by the whole block, every entry's
+//                         rank by counting), sort a copy of its out-list by
+//                         column, count the union
 //   scan                  row offsets of K'
 //   sym_rows_kernel<1>    per row: merge into K' (deterministic: both lists
 //                         sorted), weights 0.5 (w_pq + w_qp)
 // One thread per row; in-lists are short except at hubs, whose insertion sort
 // by one thread was the cost (60001 x 50, k = 8, in-lists up to 409: sym_rows_kernel<0>
-// 2.44 ms; with the long lists ranked before it 0.10 + 0.14 ms).
+// 2.44 ms; with the long lists ranked by blocks 0.24).  Ranked in a launch of their
+// own, graphs without hubs paid 4 to 5 % for it (100000 rows, k = 8: 0.250 ms against
+// 0.239).
 #include <stdint.h>
 
 #include "slk_internal.cuh"
@@ -89,70 +91,70 @@ __global__ void sym_in_fill_kernel(const int64_t* __restrict__ row_ptr,
     }
 }
 
-// In-lists of more than kLongList entries sorted by (source, weight): a block
-// looks at 256 rows, then its threads rank the entries of each long list
-// against all of them into tmp (as long as the in-lists) and copy them back.
+// In-lists of more than kLongList entries are sorted by (source, weight) by the
+// block: its threads rank the entries of each against all of them into tmp (as
+// long as the in-lists) and copy them back.
 constexpr int kLongList = 48;
 // weights in an order that is total (NaN too), so that the ranks are a permutation
 __device__ __forceinline__ uint32_t weight_key(float w) {
     const uint32_t u = __float_as_uint(w);
     return u >> 31 ? ~u : u | 0x80000000u;
 }
-__global__ void __launch_bounds__(256)
-sym_sort_long_kernel(const int64_t* __restrict__ in_ptr, int64_t N, int32_t* in_src, float* in_w,
-                     int32_t* tmp_src, float* tmp_w) {
+// The long lists of rows p0 .. p0 + 255 (every thread of the block; tells if there are any).
+__device__ __forceinline__ void sort_long_lists(const int64_t* __restrict__ in_ptr, int64_t p0, bool is_long,
+                                                int32_t* in_src, float* in_w, int32_t* tmp_src, float* tmp_w) {
     __shared__ int list[256];
     __shared__ int n;
+    if (!__syncthreads_or(is_long)) return;
     const int t = threadIdx.x;
-    for (int64_t p0 = (int64_t)blockIdx.x * 256; p0 < N; p0 += (int64_t)gridDim.x * 256) {
-        __syncthreads();
-        if (t == 0) n = 0;
-        __syncthreads();
-        if (p0 + t < N && in_ptr[p0 + t + 1] - in_ptr[p0 + t] > kLongList) list[atomicAdd(&n, 1)] = t;
-        __syncthreads();
-        for (int i = 0; i < n; ++i) {
-            const int64_t i0 = in_ptr[p0 + list[i]], i1 = in_ptr[p0 + list[i] + 1];
-            for (int64_t a = i0 + t; a < i1; a += 256) {
-                const int32_t s = in_src[a];
-                const float w = in_w[a];
-                const uint32_t k = weight_key(w);
-                int64_t r = i0;
-                for (int64_t b = i0; b < i1; ++b) {
-                    const int32_t s2 = in_src[b];
-                    if (s2 < s) ++r;
-                    else if (s2 == s && b != a) {
-                        const uint32_t k2 = weight_key(in_w[b]);
-                        r += k2 < k || (k2 == k && b < a);
-                    }
+    if (t == 0) n = 0;
+    __syncthreads();
+    if (is_long) list[atomicAdd(&n, 1)] = t;
+    __syncthreads();
+    for (int i = 0; i < n; ++i) {
+        const int64_t i0 = in_ptr[p0 + list[i]], i1 = in_ptr[p0 + list[i] + 1];
+        for (int64_t a = i0 + t; a < i1; a += 256) {
+            const int32_t s = in_src[a];
+            const float w = in_w[a];
+            const uint32_t k = weight_key(w);
+            int64_t r = i0;
+            for (int64_t b = i0; b < i1; ++b) {
+                const int32_t s2 = in_src[b];
+                if (s2 < s) ++r;
+                else if (s2 == s && b != a) {
+                    const uint32_t k2 = weight_key(in_w[b]);
+                    r += k2 < k || (k2 == k && b < a);
                 }
-                tmp_src[r] = s;
-                tmp_w[r] = w;
             }
-            __syncthreads();
-            for (int64_t a = i0 + t; a < i1; a += 256) {
-                in_src[a] = tmp_src[a];
-                in_w[a] = tmp_w[a];
-            }
-            __syncthreads();
+            tmp_src[r] = s;
+            tmp_w[r] = w;
         }
+        __syncthreads();
+        for (int64_t a = i0 + t; a < i1; a += 256) {
+            in_src[a] = tmp_src[a];
+            in_w[a] = tmp_w[a];
+        }
+        __syncthreads();
     }
 }
 
 // WRITE = 0: sort row p's in-list (by source, then weight for a repeated
 // source) and store the size of the union with its out-list in cnt[p];
-// WRITE = 1: write row p of K' from the two sorted lists.
+// WRITE = 1: write row p of K' from the two sorted lists.  256 threads.
 template <int WRITE>
 __global__ void sym_rows_kernel(const int64_t* __restrict__ row_ptr,
                                 const int32_t* __restrict__ col_idx, const float* __restrict__ w,
                                 int64_t N, const int64_t* __restrict__ in_ptr,
-                                int32_t* __restrict__ in_src, float* __restrict__ in_w,
+                                int32_t* in_src, float* in_w,
                                 int64_t* __restrict__ cnt, const int64_t* __restrict__ out_ptr,
-                                int32_t* __restrict__ out_col, float* __restrict__ out_w,
-                                unsigned int* __restrict__ err) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i0 = in_ptr[p], i1 = in_ptr[p + 1];
-        if (!WRITE && i1 - i0 <= kLongList) {   // longer ones are sorted already
+                                int32_t* out_col, float* out_w, unsigned int* __restrict__ err) {
+    for (int64_t p0 = (int64_t)blockIdx.x * 256; p0 < N; p0 += (int64_t)gridDim.x * 256) {
+        const int64_t p = p0 + threadIdx.x;
+        const int64_t i0 = p < N ? in_ptr[p] : 0, i1 = p < N ? in_ptr[p + 1] : 0;
+        // (the outputs, twice as long as the in-lists, serve as scratch)
+        if (!WRITE) sort_long_lists(in_ptr, p0, i1 - i0 > kLongList, in_src, in_w, out_col, out_w);
+        if (p >= N) continue;
+        if (!WRITE && i1 - i0 <= kLongList) {
             for (int64_t a = i0 + 1; a < i1; ++a) {   // insertion sort by (source, weight)
                 const int32_t ks = in_src[a];
                 const float kw = in_w[a];
@@ -256,12 +258,8 @@ slk_status symmetrize_launch(slk_ctx* ctx, const int64_t* row_ptr, const int32_t
     if (r != SLK_OK) return r;
     sym_in_fill_kernel<<<(unsigned)g, 256, 0, s>>>(row_ptr, col_idx, w, N, in_ptr, cursor, in_src, in_w);
     SLK_LAUNCH_CHECK(ctx, "sym_in_fill_kernel");
-    // (the outputs, twice as long as the in-lists, serve as scratch)
-    SLK_COUNT_LAUNCH(ctx, 1);
-    sym_sort_long_kernel<<<(unsigned)g, 256, 0, s>>>(in_ptr, N, in_src, in_w, out_col, out_w);
-    SLK_LAUNCH_CHECK(ctx, "sym_sort_long_kernel");
     sym_rows_kernel<0><<<(unsigned)g, 256, 0, s>>>(row_ptr, col_idx, w, N, in_ptr, in_src, in_w, cnt,
-                                                   nullptr, nullptr, nullptr, err);
+                                                   nullptr, out_col, out_w, err);
     SLK_LAUNCH_CHECK(ctx, "sym_rows_kernel<0>");
     r = scan_launch(ctx, cnt, N, out_row_ptr, btot);
     if (r != SLK_OK) return r;
