@@ -212,7 +212,7 @@ struct DensItem {
     int32_t slot;         // row of the partial-sum matrix
 };
 
-// 128 (or fewer) consecutive places of one cluster.
+// Consecutive places of one cluster inside one block of 128 places.
 struct DensRows {
     int32_t label, row0, row1;
 };
@@ -228,20 +228,29 @@ struct DensSmem {
 };
 
 // Grid: (row blocks, items).  Thread (ty, tx) = (t / 16, t % 16) owns rows
-// {4ty..4ty+3, 64+4ty..+3} and the same pattern of columns.  other: 0 the
-// row blocks of the item's own cluster, 1 those of the others that need it.
+// {4ty..4ty+3, 64+4ty..+3} and the same pattern of columns.  rows given: the
+// pieces of the item's own cluster; NULL: the blocks of 128 places that need it,
+// whole, so that none of a tile's rows idle where clusters are small (where a block
+// holds rows of the item's own cluster too, their sums are written again).
+// 100000 x 32 points of one cluster, L = 100, nothing to leave out: 31.8 ms with
+// every block cut at the clusters, now 30.2 (30.0 for one pass over all pairs).
 __global__ void __launch_bounds__(DT, 2)
 density_tile_kernel(const float* __restrict__ xt, const float* __restrict__ norms, int64_t N,
                     int Dp, const int32_t* __restrict__ perm, const DensRows* __restrict__ rows,
-                    const DensItem* __restrict__ items, int other, const uint8_t* __restrict__ need, int L,
+                    const DensItem* __restrict__ items, const uint8_t* __restrict__ need, int L,
                     const float* __restrict__ sigma_dev, double* __restrict__ part) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     DensSmem& s = *reinterpret_cast<DensSmem*>(smem_raw);
     const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
-    const DensRows rw = rows[blockIdx.x];
     const DensItem it = items[blockIdx.y];
-    if ((rw.label == it.label) == (other != 0)) return;
-    if (other && !need[(int64_t)blockIdx.x * L + it.label]) return;
+    DensRows rw;
+    if (rows) {
+        rw = rows[blockIdx.x];
+        if (rw.label != it.label) return;
+    } else {
+        if (!need[(int64_t)blockIdx.x * L + it.label]) return;
+        rw = {-1, (int)blockIdx.x * DBM, (int)min((int64_t)(blockIdx.x + 1) * DBM, N)};
+    }
     const float sg = *sigma_dev;
     const float inv2s2 = 1.0f / (2.0f * sg * sg);
     if (t < DBM) {
@@ -387,7 +396,8 @@ density_depth_kernel(const float* __restrict__ d2, const int32_t* __restrict__ p
     }
 }
 
-// need[b][l]: a row of block b (another cluster's) may reach T_l:
+// need[b][l]: a row of another cluster's in the b-th 128 places may reach T_l
+// (need starts at 0):
 // f_l(y) <= sum over cluster l's depths of exp(-(h_jl(y) + h_lj(p))^2 / 2 sigma^2).
 __global__ void __launch_bounds__(256)
 density_reach_kernel(const float* __restrict__ lo, const int* __restrict__ hist,
@@ -406,7 +416,8 @@ density_reach_kernel(const float* __restrict__ lo, const int* __restrict__ hist,
             const float r = fmaxf(y + 0.25f * (float)(k - 32) - 1e-4f, 0.f) * 0.9999f;
             f += (float)h[k] * expf(-0.5f * r * r);
         }
-        need[i] = !((double)f * 1.0001 < T);   // NaN (no border) needs it
+        if (j != l && !((double)f * 1.0001 < T))   // NaN (no border) needs it
+            need[(int64_t)(rows[b].row0 / DBM) * L + l] = 1;
     }
 }
 
@@ -677,13 +688,17 @@ slk_status init_modes_launch(slk_ctx* ctx, const float* X, int64_t N, int D, con
                                       cudaMemcpyHostToDevice, s));
     std::vector<DensRows> hrow;
     for (int l = 0; l < L; ++l)
-        for (int64_t c = hoff[l]; c < hoff[l + 1]; c += DBM)
-            hrow.push_back({l, (int32_t)c, (int32_t)std::min<int64_t>(c + DBM, hoff[l + 1])});
+        for (int64_t c = hoff[l], e; c < hoff[l + 1]; c = e) {
+            e = std::min<int64_t>((c / DBM + 1) * DBM, hoff[l + 1]);
+            hrow.push_back({l, (int32_t)c, (int32_t)e});
+        }
     const int n_rows = (int)hrow.size();
     if (n_rows > pl.max_rows) return set_err(ctx, SLK_ERR_CUDA, "density rows overflow");
     SLK_CUDA_TRY(ctx, cudaMemcpyAsync(rows, hrow.data(), sizeof(DensRows) * hrow.size(),
                                       cudaMemcpyHostToDevice, s));
     // 5. density tiles: own clusters, T_l, then the row blocks that may reach it
+    const int64_t n_blocks = (N + DBM - 1) / DBM;
+    SLK_CUDA_TRY(ctx, cudaMemsetAsync(need, 0, (size_t)n_blocks * L, s));
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(hist, 0, sizeof(int) * (size_t)L * L * kDepthBins, s));
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(tbits, 0, sizeof(unsigned long long) * (L + 1), s));
     int gx = (int)((N + 255) / 256);
@@ -695,13 +710,12 @@ slk_status init_modes_launch(slk_ctx* ctx, const float* X, int64_t N, int D, con
     SLK_COUNT_LAUNCH(ctx, 7);
     density_depth_kernel<<<(unsigned)n_rows, DBM, 0, s>>>(d2, perm, rows, seeds, L, sigma_dev, lo, hist);
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(part, 0, sizeof(double) * hit.size() * (size_t)N, s));
-    density_tile_kernel<<<tgrid, DT, smem, s>>>(xt, norms, N, pl.Dp, perm, rows, items, 0, need, L,
-                                                sigma_dev, part);
+    density_tile_kernel<<<tgrid, DT, smem, s>>>(xt, norms, N, pl.Dp, perm, rows, items, need, L, sigma_dev, part);
     density_bound_kernel<<<bgrid, 256, 0, s>>>(part, N, pl.Dp, norms, st, sigma_dev, slot0, 0, tbits, cand,
                                                ncand, pl.cand_cap);
     density_reach_kernel<<<(unsigned)gx, 256, 0, s>>>(lo, hist, rows, n_rows, L, tbits, sigma_dev, need);
-    density_tile_kernel<<<tgrid, DT, smem, s>>>(xt, norms, N, pl.Dp, perm, rows, items, 1, need, L,
-                                                sigma_dev, part);
+    density_tile_kernel<<<dim3((unsigned)n_blocks, (unsigned)hit.size()), DT, smem, s>>>(
+        xt, norms, N, pl.Dp, perm, nullptr, items, need, L, sigma_dev, part);
     SLK_LAUNCH_CHECK(ctx, "density_tile_kernel");
     // 6. candidates: upper bound of f_l(y) reaches the largest lower bound (a
     // sum that was left out is 0 and cannot)
