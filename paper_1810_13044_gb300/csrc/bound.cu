@@ -976,18 +976,28 @@ __device__ __forceinline__ float rows_update_cached(int lr0, int lstride, int nr
 // of 150001 points, L = 37, k = 7: 2.82 ms, now 2.20; 200 of 70000, L = 10,
 // k = 5: 2.00, now 1.76.  One label per lane: four rows (144 registers) hide
 // more than warps do (2000 points, L = 5: 0.052 ms; 0.087 with four blocks).
-template <int LPL>
+// FEW: small problems, whose blocks have a row or two per group: two rows and as
+// many blocks as the registers allow there too, half the blocks at the barrier.
+// 100 updates with one row and with two (ms): 4000 points, L = 9, k = 5: 0.462,
+// 0.403; k = 10: 0.538, 0.501; 20000, L = 20, k = 5: 0.832, 0.799; k = 10: 1.012,
+// 1.033; 30000, L = 33, k = 5: 1.32, 1.57.
+template <int LPL, bool FEW>
 struct CachedTiling {
-    static constexpr int rpg = (LPL == 1) ? 4 : (LPL == 4 ? 2 : 1);
-    static constexpr int blocks = (LPL == 2) ? 4 : 1;
+    static constexpr int rpg = (LPL == 1) ? 4 : (LPL == 4 || (LPL == 2 && FEW)) ? 2 : 1;
+    static constexpr int blocks = (LPL == 2 && !FEW) ? 4 : 1;
 };
+// Where FEW is the faster one: rows times lanes per row below about twice the
+// lanes that four blocks per SM have (short rows), or three quarters of them.
+bool cached_few(int64_t N, int G, int kdeg, int num_sms) {
+    return N * G * 100 <= (int64_t)(kdeg <= 5 ? 210 : 77) * 4 * kThreads * num_sms;
+}
 
 // Persistent inner loop over a fixed-degree graph (kdeg edges per row) with
 // each CTA's operands cached in shared memory: CTA b owns rows
 // [b rpc, (b + 1) rpc).  Same updates, barrier and results as
 // bound_persistent_kernel.
-template <int G, int LPL>
-__global__ void __launch_bounds__(kThreads, CachedTiling<LPL>::blocks)
+template <int G, int LPL, bool FEW>
+__global__ void __launch_bounds__(kThreads, CachedTiling<LPL, FEW>::blocks)
 bound_cached_kernel(const float* __restrict__ A, const int32_t* __restrict__ col_idx,
                     const float* __restrict__ w, int64_t N, int L, float lambda, float* Z0,
                     float* Z1, int max_iters, float tol, int kdeg, int rpc, DevState* st) {
@@ -1010,7 +1020,7 @@ bound_cached_kernel(const float* __restrict__ A, const int32_t* __restrict__ col
     const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (grp * G));
     const int gidx = warp * RPW + grp;
     constexpr int ng = (kThreads / 32) * RPW;   // groups per CTA
-    constexpr int RPG = CachedTiling<LPL>::rpg;
+    constexpr int RPG = CachedTiling<LPL, FEW>::rpg;
     int it = 0;
     while (it < max_iters) {
         const float* Zin = (it & 1) ? Z1 : Z0;
@@ -1258,12 +1268,12 @@ constexpr int64_t kStagedMinRows = 100000;     // below: the graph sits in L2, l
 // Launches bound_cached_kernel when the graph has a fixed degree and every
 // CTA's share of A, col_idx and w fits kCachedSmemMax with all CTAs resident;
 // *used says whether it did.
-template <int G, int LPL>
+template <int G, int LPL, bool FEW>
 cudaError_t launch_cached(slk_ctx* ctx, const float* A, const int32_t* col_idx, const float* w,
                           int64_t N, int L, float lambda, float* Z, float* Z_prev, int max_iters,
                           float tol, int kdeg, DevState* st, bool* used) {
     *used = false;
-    auto kern = bound_cached_kernel<G, LPL>;
+    auto kern = bound_cached_kernel<G, LPL, FEW>;
     const size_t per_row = sizeof(float) * L + sizeof(int) * kdeg + (w ? sizeof(float) * kdeg : 0);
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, 0);
@@ -1347,8 +1357,11 @@ slk_status bound_launch(slk_ctx* ctx, const float* A, const int64_t* row_ptr,
         SLK_COUNT_LAUNCH(ctx, 1);
         bool cached = false;
 #define SLK_LAUNCH_CACHED(G_, LPL_)                                                            \
-    e = launch_cached<G_, LPL_>(ctx, A, col_idx, w, N, L, lambda, Z, Z_prev, max_iters, tol,   \
-                                kdeg, st, &cached);
+    {                                                                                          \
+        auto launch = LPL_ == 2 && cached_few(N, G_, kdeg, ctx->num_sms)                       \
+                          ? launch_cached<G_, LPL_, LPL_ == 2> : launch_cached<G_, LPL_, false>; \
+        e = launch(ctx, A, col_idx, w, N, L, lambda, Z, Z_prev, max_iters, tol, kdeg, st, &cached); \
+    }
         if (kdeg > 0) SLK_DISPATCH_L(L, SLK_LAUNCH_CACHED);
 #undef SLK_LAUNCH_CACHED
         if (e != cudaSuccess) return cuda_err(ctx, e, "bound_cached_kernel");
