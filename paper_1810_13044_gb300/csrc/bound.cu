@@ -447,9 +447,13 @@ __device__ __forceinline__ float row_update_named(int64_t p, int64_t e0, int cnt
 // set of rows and a neighbour's load waiting for its name; 8.1 with names
 // ahead and hubs first, windows of 8, three blocks per SM; 7.3 with the queue;
 // 5.9 with windows of 16 and two blocks per SM (32: 6.4; four blocks: 7.3).
+// Eight lanes of two labels have windows of 8 and run three blocks per SM: 30
+// updates of such a graph (largest degree 343) at L = 10 1.51 ms, of 300000 rows
+// of about 14 edges 2.35; with two blocks 1.62 and 3.17, with windows of 16 1.38
+// and 3.07 (a fixed set of rows per group: 2.27 and 2.98).
 constexpr int kHubDeg = 48, kHubMax = 512;
 template <int G, int LPL>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, G == 8 && LPL == 2 ? 3 : 2)
 bound_var_kernel(const float* __restrict__ A, const int64_t* __restrict__ row_ptr,
                  const int32_t* __restrict__ col_idx, const float* __restrict__ w,
                  int64_t N, int L, float lambda, float* Z0, float* Z1, int max_iters,
