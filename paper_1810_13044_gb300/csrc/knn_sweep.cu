@@ -39,12 +39,15 @@
 // per scheduler its chain of dependent instructions ran at 0.15 a cycle.
 // Sweeps over every tile, the kernel with sorted lists and this one: 1.04 and
 // 0.37 ms at 19870 x 9, 2.28 and 1.17 at 42099 x 64, 3.48 and 2.30 at 60001 x 50,
-// 6.59 and 5.59 at 70000 x 784; at 1e6 x 128 it is the slower one (293 and 316
-// ms: hits cost 45 instructions each, and two lists of eight warps took them),
-// but few of those tiles are left to sweep (knn_group.cu).
+// 6.59 and 5.59 at 70000 x 784.  Points of one cluster, which leave no tile out,
+// with k = 10: 19.6 and 15.7 ms at 200000 x 128, 87 and 79 at 500000 x 128, 126 and
+// 126 at 500000 x 256, 293 and 291 at 1e6 x 128; with k = 24 hits are more (45
+// instructions each) and the eight warps that took them for the sorted lists were
+// quicker: 60.0 and 60.5 ms at 400000 x 128, 272 and 293 at 1e6 x 32.
 //
 // Every mbarrier wait is bounded in time; on a timeout the CTA raises an
 // error bit, drains its own copies in flight, frees TMEM and returns.
+#include <cstddef>
 #include <type_traits>
 
 #include "knn_cert.cuh"
@@ -55,14 +58,18 @@ namespace {
 
 enum { PLAIN = 0, AUG = 1, RES = 2, SPLIT = 3 };
 
-// Operand stages.  Where the epilogue bounds the tiles (folded norms) two, so
-// that the row buffers are 80 slots long and refreshes rare: at 200000 x 128,
-// k = 10, 5.15 ms, against 7.81 with three stages and 64 slots; 104 slots gain
-// 0.3 ms there and lose 10 % at 19870 x 9, k = 5 (longer refreshes).
+// Three operand stages and as many slots as fit beside them.  A stage's round
+// trip (copy, MMAs, release) is longer than two stages' MMAs, so with two of them
+// large sweeps waited for operands: 315 ms at 1e6 x 128 (now 291), 169 at 500000 x
+// 256 (now 126).  More and smaller stages were slower: half slices of B's features
+// (five, 64-byte rows) 367 ms at 1e6 x 128, half tiles of columns (five, N = 128)
+// 459.  Slots fewer than 76 refresh the rows too often where clusters are dense:
+// 1e6 x 128 manifolds 86.8 ms with 76, 91 with 72, 105 with 64 (87.6 with 80 and two
+// stages); 104 slots lose 10 % at 19870 x 9, k = 5 (longer refreshes).
 template <int FORM> struct Shape {
     static constexpr bool fold = FORM == AUG || FORM == RES;
-    static constexpr int stages = fold ? 2 : 3;
-    static constexpr int slots = 80;     // buffered candidates per row
+    static constexpr int stages = 3;
+    static constexpr int slots = FORM == RES ? 76 : 80;   // buffered candidates per row
 };
 constexpr int GRP = 8;               // columns appended between room checks
 constexpr int RES_MAX_DP = 128;
@@ -74,18 +81,32 @@ struct Smem {
     static constexpr int STAGES = Shape<FORM>::stages, SLOTS = Shape<FORM>::slots;
     uint8_t a[FORM == RES ? RES_MAX_DP / TC_BK : STAGES][A_BYTES];   // 1024-byte aligned
     uint8_t b[STAGES][B_BYTES];
-    uint8_t a_aug[FORM == RES ? AUG_A_BYTES : 16];
-    uint8_t b_aug[FORM == RES ? STAGES : 1][FORM == RES ? AUG_B_BYTES : 16];
-    float buf_d[SLOTS][TC_M];        // candidates of each row (column = row of the block)
+    // candidates of each row (column = row of the block); a refresh reads them by
+    // eights, up to four slots past the end (into what follows)
+    float buf_d[SLOTS][TC_M];
     int buf_i[SLOTS][TC_M];
+    uint8_t a_aug[FORM == RES ? AUG_A_BYTES : 16];   // 1024-byte aligned
+    uint8_t b_aug[2][FORM == RES ? AUG_B_BYTES : 16];
     unsigned long long full[STAGES], empty[STAGES], tfull[2], tempty[2], afull, aempty;
     unsigned long long colbar[8];    // tile column handed from the producer to the epilogue
     int tcol[8];
     uint32_t tmem_base;
     int abort;
 };
+static_assert(offsetof(Smem<RES>, a_aug) % 1024 == 0 && Shape<RES>::stages == 3, "folded norms");
 static_assert(sizeof(Smem<RES>) + 1024 <= 232448 && sizeof(Smem<AUG>) + 1024 <= 232448 &&
               sizeof(Smem<PLAIN>) + 1024 <= 232448, "shared memory");
+
+// Place of a tile's folded norms (RES).  A slot is free again when the stage of
+// a later tile's last slice is: with two slices a tile and three stages that
+// stage's last MMAs were those of the tile in between, so two slots are enough;
+// with one slice it takes as many as stages, the last in A's second slice, which
+// such a form does not use.
+template <int FORM>
+__device__ __forceinline__ uint8_t* aug_slot(Smem<FORM>& s, int nkb0, uint32_t stage, uint32_t tile) {
+    const uint32_t i = nkb0 == 1 ? stage : tile & 1u;
+    return i == 2u ? s.a[1] : s.b_aug[i];
+}
 
 struct SweepArgs {
     SweepWork w;
@@ -267,6 +288,9 @@ __device__ __noinline__ RowState refresh(float* d, int* idx, RowState s, int k, 
     s.cnt = n;
     return s;
 }
+// A refresh cuts a list of more than FULL entries to at most KEEP, so that the
+// buffer has room for some 20 more (with KEEP = 60 fewer rows stay open, but it
+// fills again after about ten).
 constexpr int FULL = 54, KEEP = 52;
 
 template <int FORM>
@@ -371,10 +395,11 @@ knn_sweep_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         const uint32_t st = iter % STAGES, use = iter / STAGES;
                         if (use > 0 && !(ok = mbar_wait(&s.empty[st], (use - 1) & 1, abort))) break;
                         if constexpr (FORM == RES) {
+                            // the last slice with the tile's folded norms
                             const bool last = kb == nkb0 - 1;
                             mbar_expect_tx(&s.full[st], B_BYTES + (last ? AUG_B_BYTES : 0u));
                             tma_load_2d(s.b[st], &tmB, &s.full[st], kb * TC_BK, bcol);
-                            if (last) tma_load_2d(s.b_aug[st], &tmB2, &s.full[st], 16, bcol);
+                            if (last) tma_load_2d(aug_slot(s, nkb0, st, tseq - 1), &tmB2, &s.full[st], 16, bcol);
                         } else if (FORM == AUG && kb == nkb0) {
                             // the folded norms: 16 columns of A (x = 0) and B (x = 16)
                             mbar_expect_tx(&s.full[st], AUG_A_BYTES + AUG_B_BYTES);
@@ -450,7 +475,7 @@ knn_sweep_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                      (kb | k) != 0 ? 1u : 0u);
                             if (FORM == RES && kb == nkb0 - 1)
                                 umma(d_tmem, sw32_desc(su32(s.a_aug)),
-                                     sw32_desc(su32(s.b_aug[FORM == RES ? st : 0])), 1u);
+                                     sw32_desc(su32(aug_slot(s, nkb0, st, tcount))), 1u);
                         }
                         umma_commit(&s.empty[st]);
                         ++iter;
