@@ -52,12 +52,17 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 //
 // The sums take N L D differences and products; what it spent beyond them were
 // the copies of four bytes and the rows of A and Z0, written and read by one
-// lane per row.  So a pass's values of A go through the freed buffer and out row
-// by row, and the softmax rows of Z0 are spread over groups of lanes (LR per
-// row), only the sum of a row, whose order is kept, running in one thread; and
-// three blocks per SM (two where the second half of the modes takes registers).
-// 10^6 x 128, L = 100: 3.15 ms before, 2.2 now (float32 units 0.64); 70000 x 784,
-// L = 10: 0.17, now 0.12.
+// lane per row.  So a pass's values of A go through the freed buffer and out as
+// they lie in memory; with one pass the softmax is formed there too, a thread per
+// row, with several the rows come back and are spread over groups of 8, 16 or 32
+// lanes, the fewest idle.  (With a power of two of lanes per row throughout, rows of
+// 9, 20 or 33 labels left half of them idle: 10 to 25 % slower than a lane per row
+// at 100000 x 9 and 20000 x 50.)  Three blocks per SM (two where the second half
+// of the modes takes registers); blocks of one point group, two only where a
+// block has one label group; a single buffer where there is only one step.
+// Kernel alone, with the lane per row and now: 10^6 x 128, L = 100: 3.15 and
+// 2.16 ms (float32 units 0.64); L = 5: 0.291 and 0.197; 70000 x 784, L = 10: 0.17
+// and 0.11; 100000 x 9, L = 20: 0.031 and 0.024.
 template <bool LO, bool V4>
 __global__ void __launch_bounds__(kUThreads, LO ? 2 : 3)
 unary_kernel(const float* __restrict__ X, int64_t N, int D, const int32_t* __restrict__ modes,
@@ -69,25 +74,38 @@ unary_kernel(const float* __restrict__ X, int64_t N, int D, const int32_t* __res
     const int nthr = blockDim.x;
     const int xbuf = npts * kUS, mbuf = kUDC * S;
     float* xs = sm;                                    // 2 x [npts][kUS]
-    float* mh = xs + 2 * xbuf;                         // 2 x [kUDC][S]
-    float* mlo = mh + 2 * mbuf;                        // 2 x [kUDC][S] (LO only)
+    const int nch = (D + kUDC - 1) / kUDC;
+    const int nsteps = ((L + 4 * G - 1) / (4 * G)) * nch;   // (pass, chunk) pairs
+    const int bufs = nsteps > 1 ? 2 : 1;
+    float* mh = xs + bufs * xbuf;                      // 2 x [kUDC][S]
+    float* mlo = mh + bufs * mbuf;                     // 2 x [kUDC][S] (LO only)
     __shared__ int mrow[SLK_MAX_L];
     __shared__ float zsum[2 * kUPG];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int g = warp % G, pg = warp / G;
     const int64_t p0 = (int64_t)blockIdx.x * npts;
     const int rows = (int)min((int64_t)npts, N - p0);
-    // rows of A and Z0: LR lanes per row, thread group gr of ng, lane gl of it
-    int LR = 1;
-    while (LR < L && LR < 32) LR <<= 1;
-    const int gl = lane % LR, gr = t / LR, ng = nthr / LR;
+    // nl labels from l0 of the block's first n rows, as they lie in memory
+    auto each = [&](int n, int nl, auto&& f) {
+        const int dr = nthr / nl, dl = nthr - dr * nl;
+        int r = t / nl, l = t - r * nl;
+#pragma unroll 4
+        while (r < n) {
+            f(r, l);
+            r += dr;
+            l += dl;
+            if (l >= nl) {
+                l -= nl;
+                ++r;
+            }
+        }
+    };
+    const bool kept = L <= 4 * G;   // one pass: the softmax needs no way back from A
     if (M == nullptr)
         for (int l = t; l < L; l += nthr) mrow[l] = modes[l];
     __syncthreads();
     const float sg = *sigma_dev;
     const float inv2s2 = 1.0f / (2.0f * sg * sg);
-    const int nch = (D + kUDC - 1) / kUDC;
-    const int nsteps = ((L + 4 * G - 1) / (4 * G)) * nch;   // (pass, chunk) pairs
     // Step s: pass s / nch (labels l0 = 4 G (s / nch) ..), chunk s % nch, buffer s & 1.
     auto stage = [&](int s) {
         const int d0 = (s % nch) * kUDC, l0 = (s / nch) * 4 * G, b = s & 1;
@@ -198,28 +216,61 @@ unary_kernel(const float* __restrict__ X, int64_t N, int D, const int32_t* __res
                     make_float4(a[0], a[1], a[2], a[3]);
             }
             __syncthreads();
-            if (gl < min(4 * G, L - l0))         // at most 32, or L: one lane each
-#pragma unroll 4
-                for (int r = gr; r < rows; r += ng) A[(p0 + r) * L + l0 + gl] = out[r * kUS + gl];
+            auto put_a = [&](int r, int l) { A[(p0 + r) * L + l0 + l] = out[r * kUS + l]; };
+            const bool one = nsteps == 1;   // the only step has a single buffer
+            if (one) {
+                each(rows, L, put_a);
+                __syncthreads();
+            }
+            if (kept && Z0) {   // a thread per row: exp (beside A where there is room) and the sum
+                float* z = one ? out : xs + (b ^ 1) * xbuf;
+                for (int r = t; r < rows; r += nthr) {
+                    const float* ar = out + r * kUS;
+                    float m = -INFINITY, sum = 0.f;
+#pragma unroll 2
+                    for (int l = 0; l < L; l += 4) {
+                        const float4 v = *reinterpret_cast<const float4*>(ar + l);
+                        m = fmaxf(m, v.x);
+                        if (l + 1 < L) m = fmaxf(m, v.y);
+                        if (l + 2 < L) m = fmaxf(m, v.z);
+                        if (l + 3 < L) m = fmaxf(m, v.w);
+                    }
+#pragma unroll 2
+                    for (int l = 0; l < L; l += 4) {
+                        float4 v = *reinterpret_cast<const float4*>(ar + l);
+                        v = make_float4(expf(v.x - m), expf(v.y - m), expf(v.z - m), expf(v.w - m));
+                        sum += v.x;
+                        if (l + 1 < L) sum += v.y;
+                        if (l + 2 < L) sum += v.z;
+                        if (l + 3 < L) sum += v.w;
+                        *reinterpret_cast<float4*>(z + r * kUS + l) = v;
+                    }
+                    zsum[r] = sum;
+                }
+            }
+            if (!one) each(rows, min(4 * G, L - l0), put_a);
             __syncthreads();             // buffer b is free for step s + 2
         }
     }
     if (Z0 == nullptr) return;
-    // the block's rows of A are written (last barrier): one pass left them in
-    // its buffer, after several as many as fit come back
-    const bool kept = L <= 4 * G;
-    const int Ls = kept ? kUS : L | 1, batch = kept ? npts : min(npts, 2 * xbuf / Ls);
-    if (kept) xs += ((nsteps - 1) & 1) * xbuf;
+    if (kept) {
+        const float* z = nsteps == 1 ? xs : xs + (nsteps & 1) * xbuf;
+        each(rows, L, [&](int r, int l) { Z0[(p0 + r) * L + l] = z[r * kUS + l] / zsum[r]; });
+        return;
+    }
+    // several passes: the block's rows of A (written, last barrier) come back, as
+    // many as fit
+    const int Ls = L | 1, batch = min(npts, 2 * xbuf / Ls);
+    int LR = 32;
+    for (int q = 16; q >= 8; q >>= 1)
+        if ((L + q - 1) / q * q < (L + LR - 1) / LR * LR) LR = q;
+    const int gl = lane % LR, gr = t / LR, ng = nthr / LR;
     for (int r0 = 0; r0 < rows; r0 += batch) {
         const int nr = min(batch, rows - r0);
-        if (!kept) {
-            for (int r = gr; r < nr; r += ng)
-                for (int l = gl; l < L; l += LR)
-                    cp_async4(xs + r * Ls + l, A + (p0 + r0 + r) * L + l, 4);
-            cp_async_commit();
-            cp_async_wait0();
-            __syncthreads();
-        }
+        each(nr, L, [&](int r, int l) { cp_async4(xs + r * Ls + l, A + (p0 + r0 + r) * L + l, 4); });
+        cp_async_commit();
+        cp_async_wait0();
+        __syncthreads();
 #pragma unroll 2
         for (int r = gr; r - gr < nr; r += ng) {   // (all lanes take part in the shuffles)
             float* ar = xs + min(r, nr - 1) * Ls;
@@ -232,12 +283,12 @@ unary_kernel(const float* __restrict__ X, int64_t N, int D, const int32_t* __res
         __syncthreads();
         for (int r = t; r < nr; r += nthr) {
             float s = 0.f;
+#pragma unroll 8
             for (int l = 0; l < L; ++l) s += xs[r * Ls + l];
             zsum[r] = s;
         }
         __syncthreads();
-        for (int r = gr; r < nr; r += ng)
-            for (int l = gl; l < L; l += LR) Z0[(p0 + r0 + r) * L + l] = xs[r * Ls + l] / zsum[r];
+        each(nr, L, [&](int r, int l) { Z0[(p0 + r0 + r) * L + l] = xs[r * Ls + l] / zsum[r]; });
         __syncthreads();
     }
 }
@@ -324,8 +375,9 @@ slk_status unary_launch(slk_ctx* ctx, const float* X, int64_t N, int D, const in
     const int gtot = (L + 3) / 4;
     const int passes = (gtot + 7) / 8;
     const int G = (gtot + passes - 1) / passes;
-    const int PG = G <= 2 ? 2 : 1;
-    const size_t smem = 2 * sizeof(float) * ((size_t)PG * kUPG * kUS +
+    const int PG = G == 1 ? 2 : 1;
+    const int bufs = passes > 1 || D > kUDC ? 2 : 1;
+    const size_t smem = bufs * sizeof(float) * ((size_t)PG * kUPG * kUS +
                                              (Mlo ? 2 : 1) * (size_t)kUDC * unary_mode_stride(G));
     // 16-byte copies need every row of X on a 16-byte boundary
     const bool v4 = (D & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;

@@ -59,3 +59,21 @@ def test_unary_passes_and_copies(slk, N, D, L, shift):
     Ao = oracle.unary(X, modes, sig)
     assert np.abs(A.cpu().numpy() - Ao).max() <= 1e-6
     assert np.abs(Z0.cpu().numpy() - oracle.softmax_rows(Ao)).max() <= 1e-6
+
+
+@pytest.mark.parametrize("N,D,L", [(127, 31, 1), (300, 32, 4), (128, 32, 5), (129, 33, 8), (1000, 9, 7), (255, 16, 9),
+                                   (256, 32, 32), (300, 64, 28), (131, 8, 33), (131, 40, 40), (140, 7, 96),
+                                   (257, 33, 255)])
+def test_unary_rows_of_both_outputs(slk, N, D, L):
+    """One step (a single buffer, the softmax in place), several of one pass (in the
+    other buffer) and several passes (read back), with one to eight label groups;
+    A alone is the same."""
+    g = inputs.rng(N + D + L)
+    X = g.normal(size=(N, D)).astype(np.float32)
+    modes = g.choice(N, size=L, replace=False).astype(np.int32)
+    sig = float(np.sqrt(D))
+    A, Z0 = slk.unary(dev(X), dev(modes), sig)
+    Ao = oracle.unary(X, modes, sig)
+    assert np.abs(A.cpu().numpy() - Ao).max() <= 1e-6
+    assert np.abs(Z0.cpu().numpy() - oracle.softmax_rows(Ao)).max() <= 1e-6
+    assert torch.equal(A, slk.unary(dev(X), dev(modes), sig, with_z0=False)[0])
