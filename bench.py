@@ -50,13 +50,15 @@ FP32_LANES_PER_SM = 128      # FP32 FMA units per SM (4 sub-partitions x 32)
 SEED = 1810
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of
-# a kernel on a workload, from a one-pass ncu capture, with the SHA-256 of the
-# kernel's source file at capture time: a changed source reports null.
+# a kernel on a workload, from a one-pass ncu capture, with the SHA-256 at capture
+# time of the kernel's own part of its source file, from the line that begins it
+# to the end of the kernel: a changed kernel reports null.
 NCU_TRAFFIC = {
     ("bound_staged_kernel", "manifolds_1000000x128_L100"): {
         "bytes": 6510319872 + 2380906240,
         "source": "paper_1810_13044_gb300/csrc/bound.cu",
-        "sha256": "f63b3eeed3ba7913966ecc82d97bda02d0899ec065349cc2357b2128bb16b9db",
+        "begin": "// ------------------------------------- staged form for large N",
+        "sha256": "165c1bbdfebb48dffb55511dd7dd8fbf69aa9587daa23efcadb476c7a59ec108",
     },
 }
 
@@ -76,9 +78,12 @@ def ncu_traffic(kernel, workload):
     path = os.path.join(ROOT, rec["source"])
     if not os.path.exists(path):
         return None
-    with open(path, "rb") as f:
-        if hashlib.sha256(f.read()).hexdigest() != rec["sha256"]:
-            return None
+    with open(path) as f:
+        text = f.read()
+    at = text.find(rec["begin"])
+    end = text.find("\n}\n", text.find(kernel + "(", max(at, 0)))
+    if at < 0 or end < 0 or hashlib.sha256(text[at:end].encode()).hexdigest() != rec["sha256"]:
+        return None
     return rec["bytes"]
 
 

@@ -54,3 +54,12 @@ def test_reference_arm_two_ranks_rank0_alone_prints():
     lines = _json_lines(r.stdout)
     assert len(lines) == 1, r.stdout[-2000:]
     _check_line(lines[0], 2, "mnist_like_70000x784_L10")
+
+
+def test_traffic_records_match_their_kernels():
+    """A recorded DRAM traffic is reported as long as its kernel is unchanged, and
+    is not kept beyond that."""
+    sys.path.insert(0, ROOT)
+    import bench
+    for (kernel, workload), rec in bench.NCU_TRAFFIC.items():
+        assert bench.ncu_traffic(kernel, workload) == rec["bytes"]
