@@ -1426,6 +1426,7 @@ slk_status bound_launch(slk_ctx* ctx, const float* A, const int64_t* row_ptr,
         void* args[] = {&a_, &rp_, &ci_, &w_, &n_, &l_, &lam_, &z0_, &z1_, &mi_, &tol_, &st_}; \
         e = cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)grid), dim3(kThreads), \
                                         args, 0, ctx->stream);                                 \
+        if (e != cudaSuccess) return cuda_err(ctx, e, "bound_var_kernel");                     \
         cached = true;                                                                         \
     }
         SLK_DISPATCH_L(L, SLK_LAUNCH_VAR);
