@@ -49,6 +49,11 @@ __device__ __forceinline__ bool lex_less(float d, int i, float d2, int i2) {
     return d < d2 || (d == d2 && i < i2);
 }
 
+// Rows the exact rescan takes together, in registers (1: long rows).
+__host__ __device__ __forceinline__ int exact_rows(int D) {
+    const int dpl = (D + 31) / 32;
+    return dpl <= 4 ? 16 : dpl <= 8 ? 8 : dpl <= 16 ? 4 : dpl <= 32 ? 2 : 1;
+}
 // Open rows at or below this count skip the float32 tiles (whose 128-row
 // blocks they would leave mostly empty) and go to the exact scan.
 constexpr long long kExactDirectRows = 256;
@@ -67,15 +72,22 @@ __host__ __device__ __forceinline__ int query_splits(long long F, long long cap,
     return (int)sp;
 }
 
-// Column splits of the exact scan for F rows: partial lists of k entries per
-// (row, split), at most 1024 splits (a few open rows still fill the GPU), as
-// many as cap entries hold.
-__host__ __device__ __forceinline__ int exact_splits(long long F, long long cap, int k) {
+// Column splits of the exact scan for F rows, `together` at a time, on `ctas`
+// CTAs: one item (rows, column range) per CTA, or 16 ranges where that leaves
+// less than four, but no range below 64 columns and no more partial lists of k
+// entries per (row, split) than cap entries hold.  A split costs an item's own
+// merge and the final one k entries per row: with as many as the buffer held, at
+// most 1024, the fallback took 1.18 ms for 22 rows of 9000 x 100, k = 24 (now 0.22),
+// 3.55 for 219 rows of 9000 x 900, k = 6 (0.56), 11.0 for 762 after 9000 float32
+// rows there (8.7).
+__host__ __device__ __forceinline__ int exact_splits(long long F, int together, int ctas, int64_t N,
+                                                     long long cap, int k) {
     if (F <= 0) return 1;
-    long long sp = cap / (F * (long long)k);
-    if (sp > 1024) sp = 1024;
-    if (sp < 1) sp = 1;
-    return (int)sp;
+    const long long items = (F + together - 1) / together;
+    long long sp = 4 * items <= ctas ? ctas / items : 16;
+    if (sp > (N + 63) / 64) sp = (N + 63) / 64;
+    if (sp > cap / (F * (long long)k)) sp = cap / (F * (long long)k);
+    return sp < 1 ? 1 : (int)sp;
 }
 
 // -------------------------------------------------------------------- prep
@@ -1523,14 +1535,14 @@ knn_fallback_kernel(const float* __restrict__ X, int64_t N, int D, int k,
 
 // Exact rescan for long rows (D above the 32 x 32 features the batched form
 // keeps in registers): work items (one failed row, one of cs =
-// exact_splits(F, cap, k) column ranges) taken persistently, so that a few
+// exact_splits of F column ranges) taken persistently, so that a few
 // rows still spread over every SM.  The row's features are staged in shared
 // memory; each of the 8 warps streams a share of the range, computing every
 // distance with exact_d2 (the same per-lane order and butterfly) and keeping
 // a register top-k (lane i holds entry i); the 8 lists are merged into the
 // (row, range) partial list at ((f cs + range) k), as the batched form does.
 __global__ void __launch_bounds__(256)
-knn_fallback_wide_kernel(const float* __restrict__ X, int64_t N, int D, int k,
+knn_fallback_wide_kernel(const float* __restrict__ X, int64_t N, int D, int k, int ctas,
                          const int32_t* __restrict__ fb_list, const long long* count_ptr,
                          long long cap, float* __restrict__ part_d, int32_t* __restrict__ part_i) {
     extern __shared__ float xs[];   // D floats: the row's features
@@ -1538,7 +1550,7 @@ knn_fallback_wide_kernel(const float* __restrict__ X, int64_t N, int D, int k,
     __shared__ int mi[8][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long count = *(const volatile long long*)count_ptr;
-    const int col_splits = exact_splits(count, cap, k);
+    const int col_splits = exact_splits(count, 1, ctas, N, cap, k);
     for (long long item = blockIdx.x; item < count * col_splits; item += gridDim.x) {
         const long long f = item / col_splits;
         const int cs = (int)(item % col_splits);
@@ -1597,7 +1609,7 @@ knn_fallback_wide_kernel(const float* __restrict__ X, int64_t N, int D, int k,
 }
 
 // Batched exact rescan of the rows that failed the certificate.  Work items
-// (R failed rows, one of cs = exact_splits(F, cap, k) column ranges) are
+// (R failed rows, one of cs = exact_splits of F column ranges) are
 // taken persistently, so the grid does not depend on the count F.  The R
 // rows' features are cached in registers, lane-strided like exact_d2; each
 // of the block's 8 warps streams a share of the column range once for all R
@@ -1608,7 +1620,7 @@ knn_fallback_wide_kernel(const float* __restrict__ X, int64_t N, int D, int k,
 // ((f cs + range) k).
 template <int R, int DPL>
 __global__ void __launch_bounds__(256)
-knn_fallback_batch_kernel(const float* __restrict__ X, int64_t N, int D, int k,
+knn_fallback_batch_kernel(const float* __restrict__ X, int64_t N, int D, int k, int ctas,
                           const int32_t* __restrict__ fb_list, const long long* count_ptr,
                           long long cap, float* __restrict__ part_d,
                           int32_t* __restrict__ part_i) {
@@ -1617,7 +1629,7 @@ knn_fallback_batch_kernel(const float* __restrict__ X, int64_t N, int D, int k,
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long count = *(const volatile long long*)count_ptr;
     const long long nbatch = (count + R - 1) / R;
-    const int col_splits = exact_splits(count, cap, k);
+    const int col_splits = exact_splits(count, R, ctas, N, cap, k);
     for (long long item = blockIdx.x; item < nbatch * col_splits; item += gridDim.x) {
         const long long b = item / col_splits;
         const int cs = (int)(item % col_splits);
@@ -1725,18 +1737,19 @@ knn_fallback_batch_kernel(const float* __restrict__ X, int64_t N, int D, int k,
     }
 }
 
-// Merge the partial lists of every failed row (cs = exact_splits(F, cap, k)
+// Merge the partial lists of every failed row (cs = exact_splits of F
 // of k entries at ((f cs) k)) into its k nearest: chunks of 7 entries per
 // lane beside the running k best (lane i holds entry i), k rounds of a warp
 // minimum per chunk.
 __global__ void __launch_bounds__(256)
-knn_fallback_merge_kernel(int k, const int32_t* __restrict__ fb_list, const long long* count_ptr,
+knn_fallback_merge_kernel(int64_t N, int together, int ctas, int k,
+                          const int32_t* __restrict__ fb_list, const long long* count_ptr,
                           long long cap, const float* __restrict__ part_d,
                           const int32_t* __restrict__ part_i, int32_t* __restrict__ col_idx,
                           float* __restrict__ dist2) {
     const int lane = threadIdx.x & 31;
     const long long count = *(const volatile long long*)count_ptr;
-    const int col_splits = exact_splits(count, cap, k);
+    const int col_splits = exact_splits(count, together, ctas, N, cap, k);
     const int total = col_splits * k;
     const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t f = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); f < count;
@@ -2259,8 +2272,8 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
             SLK_COUNT_LAUNCH(ctx, 2);
             const unsigned grid = (unsigned)(ctx->num_sms * 2);
 #define SLK_FB(R_, DPL_)                                                                     \
-    knn_fallback_batch_kernel<R_, DPL_><<<grid, 256, 0, s>>>(X, N, D, k, exact_list, exact_count, \
-                                                             cap, cand_d, cand_i)
+    knn_fallback_batch_kernel<R_, DPL_><<<grid, 256, 0, s>>>(X, N, D, k, (int)grid, exact_list, \
+                                                             exact_count, cap, cand_d, cand_i)
             if (dpl <= 4) SLK_FB(16, 4);
             else if (dpl <= 8) SLK_FB(8, 8);
             else if (dpl <= 16) SLK_FB(4, 16);
@@ -2268,7 +2281,8 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
 #undef SLK_FB
             SLK_LAUNCH_CHECK(ctx, "knn_fallback_batch_kernel");
             knn_fallback_merge_kernel<<<(unsigned)(ctx->num_sms * 2), 256, 0, s>>>(
-                k, exact_list, exact_count, cap, cand_d, cand_i, col_idx, dist2);
+                N, exact_rows(D), (int)grid, k, exact_list, exact_count, cap, cand_d, cand_i, col_idx,
+                dist2);
             SLK_LAUNCH_CHECK(ctx, "knn_fallback_merge_kernel");
         } else if ((size_t)D * sizeof(float) <= kWideSmemMax) {
             // long rows: staged in shared memory, (row, column range) items
@@ -2276,11 +2290,12 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
             const int smem = (int)((size_t)D * sizeof(float));
             SLK_CUDA_TRY(ctx, cudaFuncSetAttribute(knn_fallback_wide_kernel,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            knn_fallback_wide_kernel<<<(unsigned)(ctx->num_sms * 4), 256, smem, s>>>(
-                X, N, D, k, exact_list, exact_count, cap, cand_d, cand_i);
+            const int grid = ctx->num_sms * 4;
+            knn_fallback_wide_kernel<<<(unsigned)grid, 256, smem, s>>>(
+                X, N, D, k, grid, exact_list, exact_count, cap, cand_d, cand_i);
             SLK_LAUNCH_CHECK(ctx, "knn_fallback_wide_kernel");
             knn_fallback_merge_kernel<<<(unsigned)(ctx->num_sms * 2), 256, 0, s>>>(
-                k, exact_list, exact_count, cap, cand_d, cand_i, col_idx, dist2);
+                N, 1, grid, k, exact_list, exact_count, cap, cand_d, cand_i, col_idx, dist2);
             SLK_LAUNCH_CHECK(ctx, "knn_fallback_merge_kernel");
         } else {
         SLK_COUNT_LAUNCH(ctx, 1);

@@ -77,3 +77,24 @@ def test_unary_rows_of_both_outputs(slk, N, D, L):
     assert np.abs(A.cpu().numpy() - Ao).max() <= 1e-6
     assert np.abs(Z0.cpu().numpy() - oracle.softmax_rows(Ao)).max() <= 1e-6
     assert torch.equal(A, slk.unary(dev(X), dev(modes), sig, with_z0=False)[0])
+
+
+@pytest.mark.parametrize("N,D,k", [(81, 5, 24), (130, 100, 7), (1000, 128, 24), (3001, 200, 10), (2500, 300, 24),
+                                   (2000, 900, 6), (1500, 1100, 24)])
+@pytest.mark.parametrize("groups", [1, 3, 5])
+@pytest.mark.parametrize("precision", ["bf16_rerank", "fp32"])
+def test_few_rows_rescanned(slk, N, D, k, groups, precision):
+    """Points with 79 copies: their neighbours tie at distance 0, so no list certifies
+    them and they are rescanned exactly, fewer rows than CTAs, a row's columns over
+    one range or many.  Integer coordinates: the oracle's graph entry by entry."""
+    g = inputs.rng(N + D)
+    X = g.integers(0, 4, size=(N, D)).astype(np.float32)
+    groups = min(groups, N // 80)
+    at = g.permutation(N)[: 80 * groups].reshape(groups, 80)
+    for a in at:
+        X[a] = X[a[0]]
+    o_idx, o_d2 = oracle.knn(X, k)
+    gr = slk.knn_graph(dev(X), k, precision=precision)
+    assert gr.stage_rows[2] >= 80 * groups
+    np.testing.assert_array_equal(gr.col_idx.cpu().numpy().reshape(N, k), o_idx)
+    np.testing.assert_array_equal(gr.dist2.cpu().numpy().reshape(N, k).astype(np.float64), o_d2)
