@@ -15,8 +15,9 @@
 //                        float32 added in float64; first every cluster against
 //                        itself, which gives a lower bound T_l of max f_l, then
 //                        the row blocks of other clusters that may still reach
-//                        T_l (density_reach_kernel).  For a row y of cluster j
-//                        and a point p of cluster l, the signed distances
+//                        T_l (density_reach_kernel; small sets: all pairs at
+//                        once).  For a row y of cluster j and a point p of cluster
+//                        l, the signed distances
 //                          h_jl(x) = (||x - s_l||^2 - ||x - s_j||^2) / (2 ||s_j - s_l||)
 //                        from the border between the two seeds give ||y - p|| >=
 //                        h_jl(y) + h_lj(p), so a histogram of cluster l's h_lj
@@ -97,8 +98,9 @@ seed_assign_kernel(const float* __restrict__ X, int64_t N, int D, const int32_t*
         if (l < L) dd[pl * L + l] = acc[j];
     }
     __syncthreads();
-    for (int i = t; i < 32 * L; i += 256)   // [N][L] distances for the reach bounds
-        if (p0 + i / L < N) d2out[p0 * L + i] = (float)dd[i];
+    if (d2out)   // [N][L] distances for the reach bounds
+        for (int i = t; i < 32 * L; i += 256)
+            if (p0 + i / L < N) d2out[p0 * L + i] = (float)dd[i];
     if (t < 32 && p0 + t < N) {
         int best = 0;
         double bd = dd[t * L];
@@ -231,7 +233,8 @@ struct DensSmem {
 // {4ty..4ty+3, 64+4ty..+3} and the same pattern of columns.  rows given: the
 // pieces of the item's own cluster; NULL: the blocks of 128 places that need it,
 // whole, so that none of a tile's rows idle where clusters are small (where a block
-// holds rows of the item's own cluster too, their sums are written again).
+// holds rows of the item's own cluster too, their sums are written again).  need
+// NULL: all pairs, the rows in the points' order.
 // 100000 x 32 points of one cluster, L = 100, nothing to leave out: 31.8 ms with
 // every block cut at the clusters, now 30.2 (30.0 for one pass over all pairs).
 __global__ void __launch_bounds__(DT, 2)
@@ -248,27 +251,26 @@ density_tile_kernel(const float* __restrict__ xt, const float* __restrict__ norm
         rw = rows[blockIdx.x];
         if (rw.label != it.label) return;
     } else {
-        if (!need[(int64_t)blockIdx.x * L + it.label]) return;
+        if (need && !need[(int64_t)blockIdx.x * L + it.label]) return;
         rw = {-1, (int)blockIdx.x * DBM, (int)min((int64_t)(blockIdx.x + 1) * DBM, N)};
     }
     const float sg = *sigma_dev;
     const float inv2s2 = 1.0f / (2.0f * sg * sg);
     if (t < DBM) {
-        const int y = perm[rw.row0 + t < rw.row1 ? rw.row0 + t : rw.row0];
+        const int i = rw.row0 + t < rw.row1 ? rw.row0 + t : rw.row0, y = rows || need ? perm[i] : i;
         s.ridx[t] = y;
         s.nrow[t] = norms[y];
         s.rowsum[t] = 0.0;
     }
-    __syncthreads();
     const int nk = Dp / DBK;
     const int lr0 = t & 127, lq0 = t >> 7, lq1 = lq0 + 2;
     for (int c0 = it.col0; c0 < it.col1; c0 += DBN) {
-        __syncthreads();  // previous tile done with ncol / cidx / buffers
-        if (t < DBN) {
-            const int c = c0 + t;
+        if (c0 > it.col0) __syncthreads();  // previous tile done with ncol / cidx / buffers
+        if (t >= DT - DBN) {   // (the other threads load the rows' names meanwhile)
+            const int i = t - (DT - DBN), c = c0 + i;
             const int q = perm[c < it.col1 ? c : it.col0];
-            s.cidx[t] = (c < it.col1) ? q : -1;
-            s.ncol[t] = norms[q];
+            s.cidx[i] = (c < it.col1) ? q : -1;
+            s.ncol[i] = norms[q];
         }
         __syncthreads();
         float acc[8][8];
@@ -352,7 +354,7 @@ density_tile_kernel(const float* __restrict__ xt, const float* __restrict__ norm
 // every seed l: lo[b][l] = min_y h_jl(y), and hist[j][l], the cluster's points
 // by their depth in quarters of sigma (place k: at least (k - 32) / 4 sigma,
 // place 0: nothing is known).  d2 [N][L]: squared distances to the seeds
-// (within 4e-6).
+// (within 4e-6).  Grid: (row blocks, up to 8 seeds each).
 constexpr int kDepthBins = 64;
 __global__ void __launch_bounds__(DBM)
 density_depth_kernel(const float* __restrict__ d2, const int32_t* __restrict__ perm,
@@ -367,7 +369,7 @@ density_depth_kernel(const float* __restrict__ d2, const int32_t* __restrict__ p
     const float dj = d2[y * L + j], inv = 4.f / *sigma_dev;
     if (t < kDepthBins) bins[t] = 0;
     __syncthreads();
-    for (int l = 0; l < L; ++l) {
+    for (int l = blockIdx.y; l < L; l += gridDim.y) {
         const float dl = d2[y * L + l], ds = d2[(int64_t)seeds[l] * L + j];
         // without a border, and where a squared distance overflows float32 (inf -
         // inf, finite / inf), nothing is known
@@ -560,6 +562,7 @@ struct InitPlan {
     int max_items;
     int max_rows;     // row blocks of 128 places, cut at the clusters
     int64_t cand_cap; // candidates kept in a list; more means every (y, l) is recomputed
+    bool reach;       // own clusters first, then the row blocks that may reach T_l
 };
 
 InitPlan init_plan(int64_t N, int D, int L) {
@@ -574,6 +577,13 @@ InitPlan init_plan(int64_t N, int D, int L) {
     p.max_items = (int)((N + p.chunk - 1) / p.chunk) + L;
     p.max_rows = (int)(tiles + L);
     p.cand_cap = std::min<int64_t>((int64_t)N * L, (int64_t)1 << 22);
+    // The bounds' launches, the second pass and its part empty tiles pay from some
+    // work and cluster size on (a pair takes about as long as 28 features and Dp more).
+    // One pass and two, in ms, clustered points and (one cluster): 9000 x 300, L = 10:
+    // 1.56, 1.72 (1.73, 2.72); 14000 x 64, L = 200: 2.41, 1.75 (2.60, 3.09); 14000 x 300,
+    // L = 10: 3.18, 2.22 (3.12, 3.78); 22000 x 64, L = 40: 2.49, 1.29 (2.58, 2.91);
+    // 22000 x 300, L = 40: 7.54, 3.45 (7.86, 8.67)
+    p.reach = (double)N * (double)N * (p.Dp + 28) > 4e10 && N >= 500 * (int64_t)L;
     return p;
 }
 
@@ -645,7 +655,7 @@ slk_status init_modes_launch(slk_ctx* ctx, const float* X, int64_t N, int D, con
         auto kern = seed_assign_kernel<LPT_>;                                                   \
         SLK_CUDA_TRY(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                                (int)smem));                                     \
-        kern<<<grid, 256, smem, s>>>(X, N, D, seeds, L, assign, d2);                                \
+        kern<<<grid, 256, smem, s>>>(X, N, D, seeds, L, assign, pl.reach ? d2 : nullptr);           \
     }
         if (lpt <= 1) { SLK_ASSIGN(1) }
         else if (lpt <= 2) { SLK_ASSIGN(2) }
@@ -687,35 +697,41 @@ slk_status init_modes_launch(slk_ctx* ctx, const float* X, int64_t N, int D, con
     SLK_CUDA_TRY(ctx, cudaMemcpyAsync(slot0, hslot.data(), sizeof(int32_t) * (L + 1),
                                       cudaMemcpyHostToDevice, s));
     std::vector<DensRows> hrow;
-    for (int l = 0; l < L; ++l)
+    for (int l = 0; pl.reach && l < L; ++l)
         for (int64_t c = hoff[l], e; c < hoff[l + 1]; c = e) {
             e = std::min<int64_t>((c / DBM + 1) * DBM, hoff[l + 1]);
             hrow.push_back({l, (int32_t)c, (int32_t)e});
         }
     const int n_rows = (int)hrow.size();
     if (n_rows > pl.max_rows) return set_err(ctx, SLK_ERR_CUDA, "density rows overflow");
-    SLK_CUDA_TRY(ctx, cudaMemcpyAsync(rows, hrow.data(), sizeof(DensRows) * hrow.size(),
-                                      cudaMemcpyHostToDevice, s));
-    // 5. density tiles: own clusters, T_l, then the row blocks that may reach it
+    if (n_rows > 0)
+        SLK_CUDA_TRY(ctx, cudaMemcpyAsync(rows, hrow.data(), sizeof(DensRows) * hrow.size(),
+                                          cudaMemcpyHostToDevice, s));
+    // 5. density tiles: own clusters, T_l, then the row blocks that may reach it; of
+    // small sets all pairs in one pass
     const int64_t n_blocks = (N + DBM - 1) / DBM;
-    SLK_CUDA_TRY(ctx, cudaMemsetAsync(need, 0, (size_t)n_blocks * L, s));
-    SLK_CUDA_TRY(ctx, cudaMemsetAsync(hist, 0, sizeof(int) * (size_t)L * L * kDepthBins, s));
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(tbits, 0, sizeof(unsigned long long) * (L + 1), s));
     int gx = (int)((N + 255) / 256);
     if (gx > 4 * ctx->num_sms) gx = 4 * ctx->num_sms;
     const int smem = (int)sizeof(DensSmem);
     SLK_CUDA_TRY(ctx, cudaFuncSetAttribute(density_tile_kernel,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    const dim3 tgrid((unsigned)n_rows, (unsigned)hit.size()), bgrid((unsigned)gx, (unsigned)L);
-    SLK_COUNT_LAUNCH(ctx, 7);
-    density_depth_kernel<<<(unsigned)n_rows, DBM, 0, s>>>(d2, perm, rows, seeds, L, sigma_dev, lo, hist);
-    SLK_CUDA_TRY(ctx, cudaMemsetAsync(part, 0, sizeof(double) * hit.size() * (size_t)N, s));
-    density_tile_kernel<<<tgrid, DT, smem, s>>>(xt, norms, N, pl.Dp, perm, rows, items, need, L, sigma_dev, part);
-    density_bound_kernel<<<bgrid, 256, 0, s>>>(part, N, pl.Dp, norms, st, sigma_dev, slot0, 0, tbits, cand,
-                                               ncand, pl.cand_cap);
-    density_reach_kernel<<<(unsigned)gx, 256, 0, s>>>(lo, hist, rows, n_rows, L, tbits, sigma_dev, need);
+    const dim3 bgrid((unsigned)gx, (unsigned)L);
+    SLK_COUNT_LAUNCH(ctx, pl.reach ? 7 : 3);
+    if (pl.reach) {
+        SLK_CUDA_TRY(ctx, cudaMemsetAsync(need, 0, (size_t)n_blocks * L, s));
+        SLK_CUDA_TRY(ctx, cudaMemsetAsync(hist, 0, sizeof(int) * (size_t)L * L * kDepthBins, s));
+        density_depth_kernel<<<dim3((unsigned)n_rows, (unsigned)((L + 7) / 8)), DBM, 0, s>>>(
+            d2, perm, rows, seeds, L, sigma_dev, lo, hist);
+        SLK_CUDA_TRY(ctx, cudaMemsetAsync(part, 0, sizeof(double) * hit.size() * (size_t)N, s));
+        density_tile_kernel<<<dim3((unsigned)n_rows, (unsigned)hit.size()), DT, smem, s>>>(
+            xt, norms, N, pl.Dp, perm, rows, items, need, L, sigma_dev, part);
+        density_bound_kernel<<<bgrid, 256, 0, s>>>(part, N, pl.Dp, norms, st, sigma_dev, slot0, 0, tbits, cand,
+                                                   ncand, pl.cand_cap);
+        density_reach_kernel<<<(unsigned)gx, 256, 0, s>>>(lo, hist, rows, n_rows, L, tbits, sigma_dev, need);
+    }
     density_tile_kernel<<<dim3((unsigned)n_blocks, (unsigned)hit.size()), DT, smem, s>>>(
-        xt, norms, N, pl.Dp, perm, nullptr, items, need, L, sigma_dev, part);
+        xt, norms, N, pl.Dp, perm, nullptr, items, pl.reach ? need : nullptr, L, sigma_dev, part);
     SLK_LAUNCH_CHECK(ctx, "density_tile_kernel");
     // 6. candidates: upper bound of f_l(y) reaches the largest lower bound (a
     // sum that was left out is 0 and cannot)
@@ -732,9 +748,11 @@ slk_status init_modes_launch(slk_ctx* ctx, const float* X, int64_t N, int D, con
     const int64_t count = all_pairs ? (int64_t)N * L : (int64_t)hcount;
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(&st->mode_best[0], 0, sizeof(unsigned long long) * L, s));
     SLK_CUDA_TRY(ctx, cudaMemsetAsync(arg, 0x7f, sizeof(int32_t) * L, s));
-    // parts of a sum: enough blocks for the GPU when there are few candidates
+    // parts of a sum: enough blocks for the GPU when there are few candidates, none
+    // below 64 points of an average cluster
     int parts = 1;
-    while (!all_pairs && parts < 64 && count * parts < 8 * ctx->num_sms && count * 2 * parts <= pl.cand_cap)
+    while (!all_pairs && parts < 64 && count * parts < 8 * ctx->num_sms && count * 2 * parts <= pl.cand_cap &&
+           2 * parts * 64 * (int64_t)L <= N)
         parts *= 2;
     for (int pass = 0; pass < 2; ++pass) {
         for (int64_t c0 = 0; c0 < count; c0 += pl.cand_cap) {

@@ -240,7 +240,7 @@ def test_initial_modes_distances_beyond_float32(slk):
     the side of the border a point lies on.  Cluster 0 is its seed and a shell
     whose distances overflow; the shell's densest place is a point of cluster 1
     near its centre (every distance of that one, and their sums, are finite)."""
-    U, D, n = 1e19, 64, 300
+    U, D, n = 1e19, 64, 21000        # (enough work for the bounds to be used)
     sig = float(np.sqrt(0.72)) * U
     g = inputs.rng(17)
     shell = np.zeros((n, D))
@@ -256,12 +256,15 @@ def test_initial_modes_distances_beyond_float32(slk):
     d2 = np.stack([((X64 - X64[s]) ** 2).sum(1) for s in seeds], 1)
     top = float(np.finfo(np.float32).max)
     assert (d2[-n:] > top).all() and (d2[:-n].sum(1) < top).all()
-    o_modes, o_assign, o_dens = oracle.initial_modes(X, seeds, sig)
-    assert o_modes[0] == 2 and o_assign[2] == 1 and (o_assign[-n:] == 0).all()
+    assign = np.where(d2[:, 0] <= d2[:, 1], 0, 1)
+    assert assign[2] == 1 and (assign[-n:] == 0).all()
+    sample = np.concatenate([[0, 1, 2, 3], len(X) - 1 - g.choice(n, 200, replace=False)])
+    f = oracle.cluster_density(X, assign.astype(np.int32), 0, sig, sample)
+    assert f.argmax() == 2 and f[2] > 2 * np.delete(f, 2).max()
     g_modes, g_assign, g_dens = slk.initial_modes(dev(X), dev(seeds), sig)
-    np.testing.assert_array_equal(host(g_assign), o_assign)
+    np.testing.assert_array_equal(host(g_assign), assign)
     assert host(g_modes)[0] == 2
-    _check_modes(X, sig, host(g_modes), np.array(g_dens), o_modes, o_dens, o_assign)
+    assert g_dens[0] == pytest.approx(f[2], rel=DENS_RTOL)
 
 
 @pytest.mark.parametrize("D", [3, 40])
@@ -274,3 +277,31 @@ def test_kmeanspp_infinite_first_seed(slk, D):
     X[5, 1] = np.inf
     got = host(slk.kmeanspp(dev(X), 4, 5, [0.25, 0.5, 0.75]))
     np.testing.assert_array_equal(got, [5, 250, N - 1, N - 1])
+
+
+def _modes64(X, seeds, sigma):
+    """(modes, assignment, densities) over all pairs in 64 bits."""
+    Y = dev(X).double()
+    assign = torch.stack([(Y - Y[int(p)]).square().sum(1) for p in seeds], 1).argmin(1)
+    own = torch.nn.functional.one_hot(assign, len(seeds)).double()
+    Y = Y - Y.mean(0)
+    n2, f = Y.square().sum(1), []
+    for a in range(0, len(X), 2048):
+        d2 = (n2[a:a + 2048, None] + n2 - 2 * Y[a:a + 2048] @ Y.T).clamp_(min=0)
+        f.append(torch.exp(d2.mul_(-1 / (2 * sigma * sigma))) @ own)
+    dens, modes = torch.cat(f).max(0)
+    return host(modes), host(assign), host(dens)
+
+
+@pytest.mark.parametrize("N,D,L,sigma", [(30500, 5, 12, 0.3), (30500, 5, 12, 3.0), (30500, 5, 12, 40.0),
+                                         (31001, 2, 40, 0.2), (30301, 7, 1, 1.0), (14001, 200, 7, 8.0),
+                                         (30155, 16, 60, 1.0), (30140, 16, 3, 1.0)])
+def test_initial_modes_other_clusters_left_out_at_size(slk, N, D, L, sigma):
+    """The same at sizes from which the bounds are used (the last one is just below):
+    clusters of many blocks and of less than one, ends inside a block."""
+    X, _ = inputs.blobs(N=N, D=D, n_blobs=max(2, L // 2), centre_var=4.0, seed=N + L)
+    seeds = inputs.kmeanspp(X, L, seed=L)
+    o_modes, o_assign, o_dens = _modes64(X, seeds, sigma)
+    g_modes, g_assign, g_dens = slk.initial_modes(dev(X), dev(seeds), sigma)
+    _check_assign(X, seeds, host(g_assign), o_assign)
+    _check_modes(X, sigma, host(g_modes), np.array(g_dens), o_modes, o_dens, o_assign)
