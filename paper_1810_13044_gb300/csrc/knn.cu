@@ -2128,8 +2128,8 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
             knn_select_kernel<false><<<(unsigned)grid, 256, 0, s>>>(sel);
             SLK_LAUNCH_CHECK(ctx, "knn_select_kernel");
         } else {
-        // entries per lane: the splits' lists, KC each, over 32 lanes
-        const int per_lane = (pl.splits * pl.kc + 31) / 32;
+            // entries per lane: the splits' lists, KC each, over 32 lanes
+            const int per_lane = (pl.splits * pl.kc + 31) / 32;
 #define SLK_RERANK(KC_, E_)                                                                   \
     knn_rerank_kernel<KC_, 0, E_><<<(unsigned)grid, 256, 0, s>>>(                             \
         X, N, D, pl.Dp, k, pl.splits, pl.Np, cand_d, cand_i, norms, rho, gam, row_ptr, col_idx, \
@@ -2138,11 +2138,11 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
     if (per_lane <= 4) SLK_RERANK(KC_, 4);                                                    \
     else if (per_lane <= 8) SLK_RERANK(KC_, 8);                                               \
     else SLK_RERANK(KC_, 16);
-        if (pl.kc == 16) { SLK_RERANK_E(16) }
-        else { SLK_RERANK_E(32) }
+            if (pl.kc == 16) { SLK_RERANK_E(16) }
+            else { SLK_RERANK_E(32) }
 #undef SLK_RERANK_E
 #undef SLK_RERANK
-        SLK_LAUNCH_CHECK(ctx, "knn_rerank_kernel");
+            SLK_LAUNCH_CHECK(ctx, "knn_rerank_kernel");
         }
     }
     {
@@ -2157,75 +2157,75 @@ slk_status knn_graph_launch(slk_ctx* ctx, const float* X, int64_t N, int D, int 
             int32_t* fb3 = pl.two_term ? fb : fb2;   // the list that is not its input
             const long long* f32_cnt = &st->fallback_count;
             if (pl.two_term) {
-            f32_in = fb2;
-            f32_cnt = &st->fallback2_count;
-            // (a) two-term bfloat16 tiles of the open rows on the tensor cores
-            // (h . h + h . l + l . h of s = h + l, about 16 significant bits
-            // of v), the rerank under their certificate; its failures, and
-            // open rows beyond the stage's capacity, go on to (b)
-            const bool v4 = D % 4 == 0 && pl.Dp >= 128 && (reinterpret_cast<uintptr_t>(X) & 15) == 0 &&
-                            (reinterpret_cast<uintptr_t>(mu) & 15) == 0;
-            int64_t pg = (pl.Np + 7) / 8;
-            if (pg > (int64_t)ctx->num_sms * 64) pg = (int64_t)ctx->num_sms * 64;
-            SLK_COUNT_LAUNCH(ctx, 4);
-            // the operand back in the points' order where the sweep had sorted it
-            __nv_bfloat16* xh = pl.grouped ? (__nv_bfloat16*)xt : nullptr;
-            if (v4)
-                prep_split_kernel<4><<<(unsigned)pg, 256, 0, s>>>(X, N, D, pl.Dp, pl.Np, mu,
-                                                                  &st->fallback_count, xh, kb.xl16,
-                                                                  kb.norms_s, kb.rho_s, st);
-            else
-                prep_split_kernel<1><<<(unsigned)pg, 256, 0, s>>>(X, N, D, pl.Dp, pl.Np, mu,
-                                                                  &st->fallback_count, xh, kb.xl16,
-                                                                  kb.norms_s, kb.rho_s, st);
-            SLK_LAUNCH_CHECK(ctx, "prep_split_kernel");
-            int64_t gg = (pl.fcap + 7) / 8;
-            if (gg > (int64_t)ctx->num_sms * 16) gg = (int64_t)ctx->num_sms * 16;
-            gather_split_kernel<<<(unsigned)gg, 256, 0, s>>>((const __nv_bfloat16*)xt, kb.xl16, kb.norms_s,
-                                                            pl.Dp, fb, &st->fallback_count, pl.fcap,
-                                                            kb.qh, kb.ql, kb.qnorm);
-            SLK_LAUNCH_CHECK(ctx, "gather_split_kernel");
-            // dot products of 3 Dp bfloat16 products (2^-23 accumulator
-            // unit, as above), |h|, |l| within 1.004 |s| and 0.0040 |s|,
-            // plus the dropped l . l term (at most 1.016 2^-16 |s_p| |s_q|)
-            const double g3 = 3.0 * (double)pl.Dp * 1.1920928955078125e-07;
-            const double gam_s = 1.02 * g3 / (1.0 - g3) + 1.02 * 1.52587890625e-05;
-            SweepOperands op{};
-            op.a_hi = kb.qh;
-            op.a_lo = kb.ql;
-            op.b_hi = (const __nv_bfloat16*)xt;
-            op.b_lo = kb.xl16;
-            op.row_norms = kb.qnorm;
-            op.col_norms = kb.norms_s;
-            op.rho = kb.rho_s;
-            op.ids = fb;
-            op.rows_dev = &st->fallback_count;
-            op.a_rows = pl.fcap;
-            op.b_rows = pl.Np;
-            op.N = N;
-            op.D = D;
-            op.Dp = pl.Dp;
-            SweepWork swork{};
-            swork.per = swork.n_tiles = pl.n_tiles;
-            swork.row_blocks = (int)(pl.fcap / 128);
-            swork.units = pl.sunits;
-            swork.aligned = 0;
-            const SweepLists slists{kb.scand, kSweepStride};
-            slk_status r = knn_sweep_launch(ctx, op, swork, k, gam_s, slists, false, nullptr, nullptr, st);
-            if (r != SLK_OK) return r;
-            sel.w = swork;
-            sel.lists = slists;
-            sel.perm = nullptr;
-            sel.norms = kb.norms_s;
-            sel.rho = kb.rho_s;
-            sel.gam = gam_s;
-            sel.fb_list = fb2;
-            sel.fb_count = (unsigned long long*)&st->fallback2_count;
-            sel.fb_in = fb;
-            sel.count_in = &st->fallback_count;
-            sel.cap = pl.fcap;
-            knn_select_kernel<true><<<(unsigned)(ctx->num_sms * 4), 256, 0, s>>>(sel);
-            SLK_LAUNCH_CHECK(ctx, "knn_select_kernel (two-term stage)");
+                f32_in = fb2;
+                f32_cnt = &st->fallback2_count;
+                // (a) two-term bfloat16 tiles of the open rows on the tensor cores
+                // (h . h + h . l + l . h of s = h + l, about 16 significant bits
+                // of v), the rerank under their certificate; its failures, and
+                // open rows beyond the stage's capacity, go on to (b)
+                const bool v4 = D % 4 == 0 && pl.Dp >= 128 && (reinterpret_cast<uintptr_t>(X) & 15) == 0 &&
+                                (reinterpret_cast<uintptr_t>(mu) & 15) == 0;
+                int64_t pg = (pl.Np + 7) / 8;
+                if (pg > (int64_t)ctx->num_sms * 64) pg = (int64_t)ctx->num_sms * 64;
+                SLK_COUNT_LAUNCH(ctx, 4);
+                // the operand back in the points' order where the sweep had sorted it
+                __nv_bfloat16* xh = pl.grouped ? (__nv_bfloat16*)xt : nullptr;
+                if (v4)
+                    prep_split_kernel<4><<<(unsigned)pg, 256, 0, s>>>(X, N, D, pl.Dp, pl.Np, mu,
+                                                                      &st->fallback_count, xh, kb.xl16,
+                                                                      kb.norms_s, kb.rho_s, st);
+                else
+                    prep_split_kernel<1><<<(unsigned)pg, 256, 0, s>>>(X, N, D, pl.Dp, pl.Np, mu,
+                                                                      &st->fallback_count, xh, kb.xl16,
+                                                                      kb.norms_s, kb.rho_s, st);
+                SLK_LAUNCH_CHECK(ctx, "prep_split_kernel");
+                int64_t gg = (pl.fcap + 7) / 8;
+                if (gg > (int64_t)ctx->num_sms * 16) gg = (int64_t)ctx->num_sms * 16;
+                gather_split_kernel<<<(unsigned)gg, 256, 0, s>>>((const __nv_bfloat16*)xt, kb.xl16, kb.norms_s,
+                                                                pl.Dp, fb, &st->fallback_count, pl.fcap,
+                                                                kb.qh, kb.ql, kb.qnorm);
+                SLK_LAUNCH_CHECK(ctx, "gather_split_kernel");
+                // dot products of 3 Dp bfloat16 products (2^-23 accumulator
+                // unit, as above), |h|, |l| within 1.004 |s| and 0.0040 |s|,
+                // plus the dropped l . l term (at most 1.016 2^-16 |s_p| |s_q|)
+                const double g3 = 3.0 * (double)pl.Dp * 1.1920928955078125e-07;
+                const double gam_s = 1.02 * g3 / (1.0 - g3) + 1.02 * 1.52587890625e-05;
+                SweepOperands op{};
+                op.a_hi = kb.qh;
+                op.a_lo = kb.ql;
+                op.b_hi = (const __nv_bfloat16*)xt;
+                op.b_lo = kb.xl16;
+                op.row_norms = kb.qnorm;
+                op.col_norms = kb.norms_s;
+                op.rho = kb.rho_s;
+                op.ids = fb;
+                op.rows_dev = &st->fallback_count;
+                op.a_rows = pl.fcap;
+                op.b_rows = pl.Np;
+                op.N = N;
+                op.D = D;
+                op.Dp = pl.Dp;
+                SweepWork swork{};
+                swork.per = swork.n_tiles = pl.n_tiles;
+                swork.row_blocks = (int)(pl.fcap / 128);
+                swork.units = pl.sunits;
+                swork.aligned = 0;
+                const SweepLists slists{kb.scand, kSweepStride};
+                slk_status r = knn_sweep_launch(ctx, op, swork, k, gam_s, slists, false, nullptr, nullptr, st);
+                if (r != SLK_OK) return r;
+                sel.w = swork;
+                sel.lists = slists;
+                sel.perm = nullptr;
+                sel.norms = kb.norms_s;
+                sel.rho = kb.rho_s;
+                sel.gam = gam_s;
+                sel.fb_list = fb2;
+                sel.fb_count = (unsigned long long*)&st->fallback2_count;
+                sel.fb_in = fb;
+                sel.count_in = &st->fallback_count;
+                sel.cap = pl.fcap;
+                knn_select_kernel<true><<<(unsigned)(ctx->num_sms * 4), 256, 0, s>>>(sel);
+                SLK_LAUNCH_CHECK(ctx, "knn_select_kernel (two-term stage)");
             }
             // (b) float32 distance tiles of the rows still open against every
             // point, then the rerank under the float32 certificate; its

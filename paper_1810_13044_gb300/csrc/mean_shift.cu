@@ -593,9 +593,10 @@ ms_moved_kernel(const double* __restrict__ M64, const double* __restrict__ M0, i
 // features per thread in phase C, threads.  Up to 1024 features 512 threads:
 // the tile's phases are chains of shared-memory loads and shuffles between
 // barriers, and 8 warps (2 per scheduler) leave the float32 units idle four
-// fifths of the time (70000 x 784, L = 10: 8 iterations and labels:
-// 2.23 ms, now 1.78); beyond, the
-// accumulators of a thread and the rows' shared memory leave room for 256.
+// fifths of the time (70000 x 784, L = 10, 8 iterations and labels: 2.23 ms
+// with 256 threads, 1.78 with 512, 1.67 since warps without columns skip phase
+// C); beyond, the accumulators of a thread and the rows' shared memory leave
+// room for 256.
 struct MsShape {
     int R, LG, CPT, TH;
 };
