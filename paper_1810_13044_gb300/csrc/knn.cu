@@ -1814,9 +1814,9 @@ struct KnnPlan {
 
 // Sweeps shorter than this are not worth the sort's launches (0.15 to 0.2 ms).
 // Tiles per CTA times K slices and their fixed part: 490 at 19937 x 256 (0.46 ms
-// grouped, 0.47 not), 1060 at 30000 x 64 (0.43 and 0.77), 14800 at 70000 x 784
-// with 10 clusters (1.66 and 5.77; with one cluster, where nothing can be left
-// out, 6.52 and 5.81).
+// grouped, 0.47 not), 1060 at 30000 x 64 (0.47 and 0.85), 14800 at 70000 x 784
+// with 10 clusters (1.70 and 5.69; with one cluster, where nothing can be left
+// out, 6.21 and 5.65).
 constexpr int64_t kGroupMinWork = 500;
 // Tiles around a row block's own columns that the first pass takes: 4, and 8
 // from 2000 column tiles on, where regions are longer (4 against 8: 0.39 and

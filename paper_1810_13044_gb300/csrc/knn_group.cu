@@ -21,11 +21,12 @@
 // pivots.
 // Candidates of the graph (both sweeps and the passes between them), and the
 // preparation with the sort, in ms, against one sweep over every tile:
-//   70000 x 784, 10 clusters, k = 5       1.11 + 0.52    5.59 + 0.18
-//   60001 x 50, 30 clusters, k = 8        0.43 + 0.21    2.30 + 0.05
-//   200000 x 128, 100 clusters, k = 10    4.93 + 0.41   18.11 + 0.17
-//   1e6 x 128, 100 clusters, k = 10       85.5 + 1.22  315.56 + 0.67
-//   70000 x 784, one cluster, k = 5       6.00 + 0.52    5.63 + 0.18
+//   70000 x 784, 10 clusters, k = 5       1.18 + 0.52    5.50 + 0.19
+//   60001 x 50, 30 clusters, k = 8        0.44 + 0.21    2.26 + 0.05
+//   200000 x 128, 100 manifolds, k = 10   5.59 + 0.40   17.64 + 0.17
+//   1e6 x 128, 100 manifolds, k = 10      86.7 + 1.24   309.3 + 0.70
+//   70000 x 784, one cluster, k = 5       5.69 + 0.52    5.47 + 0.18
+//   1e6 x 128, one cluster, k = 10       300.2 + 1.91   291.0 + 1.35
 #include <cuda_bf16.h>
 #include <math.h>
 #include <stdint.h>
